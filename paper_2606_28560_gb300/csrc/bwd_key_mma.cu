@@ -205,7 +205,6 @@ bwd_key_mma_kernel(const __grid_constant__ RowMaps tmQ, const __grid_constant__ 
     __shared__ __align__(16) float rvals[kWarps][kMmaMaxRungs][16];
     __shared__ float wils[kWarps][32];                    // per warp: 1 / row sum of its band queries
     __shared__ float red[kMmaMaxRungs];                   // block 0: dL/dd_k
-    __shared__ long long red64[kWarps * kMmaMaxRungs];
     unsigned char* buf = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const unsigned sbase = smem_u32(buf);
 
@@ -237,7 +236,7 @@ bwd_key_mma_kernel(const __grid_constant__ RowMaps tmQ, const __grid_constant__ 
         if (pass == 1) {
             if (!waited) pdl_wait();
             waited = true;
-            if (blk == 0 && a.want_dd) convert_rung_sums(a, red, red64);
+            if (blk == 0 && a.want_dd) convert_rung_sums(a, red);
         }
         float acc[8][4];
 #pragma unroll
@@ -352,7 +351,7 @@ cudaError_t launch_nt(const RowMaps& mq, const RowMaps& mg, const BwdArgs& a, co
 
 size_t bwd_key_mma_static_smem() {
     return sizeof(float) * (kWarps * kMmaMaxRungs * 16 + kWarps * 32 + kMmaMaxRungs) +
-           sizeof(long long) * kWarps * kMmaMaxRungs + sizeof(RopeSmem) + 64;
+           sizeof(RopeSmem) + 64;
 }
 
 size_t bwd_key_mma_smem_bytes(const MmaLayout& L, bool) { return fwd_mma_smem_bytes(L); }

@@ -241,7 +241,7 @@ __device__ __forceinline__ void rope_chunk(const RopeParams& rp, int pos, int c,
 
 // dL/dd_k is the sum of the query blocks' partials.  Each block writes its
 // partials as 64-bit fixed point (2^-32 units; threads k < K hold rung k's);
-// block 0 of the key pass, which starts after the query pass has completed,
+// one block of the key pass, which waits for the query pass to complete,
 // adds them up -- integer addition is exact and order-free, so the result
 // does not depend on scheduling -- and applies the chain rule
 // dL/dalpha = sum_k f_k dL/dd_k, dL/dtheta = dL/dalpha (alpha - 0.5)(1.5 - alpha),
@@ -251,26 +251,34 @@ __device__ __forceinline__ void write_rung_partials(const BwdArgs& a, float part
         a.rpart[(size_t)threadIdx.x * a.nblk_q + blockIdx.x] = __float2ll_rn(partial * 4294967296.0f);
 }
 
-// Called by every thread of block 0 of the key pass (blockDim a multiple of
-// 32, at most 32 warps).  red: shared scratch of at least K floats; red64:
-// shared scratch of at least (blockDim / 32) * K 64-bit words.
-__device__ __forceinline__ void convert_rung_sums(const BwdArgs& a, float* red, long long* red64) {
+// Called by every thread of one block of the key pass (blockDim a multiple of
+// 32).  red: shared scratch of at least K floats.  A warp sums whole rungs,
+// kCols columns a lane in flight at a time.  Bound by load latency: one thread
+// block adds K x (query-pass blocks) words while others may already be done.
+// Rung after rung over all threads (a latency and a warp sum
+// each) it was the end of the whole backward on small grids: key pass at B1
+// H8 T1000 17.7 -> 12.5 us, at B4 22.6 -> 18.4 us, at B16 H8 Hkv2 T1024 (its
+// blocks fit one wave) 47.3 -> 41.7 us; unchanged where several waves hide it.
+__device__ __forceinline__ void convert_rung_sums(const BwdArgs& a, float* red) {
+    constexpr int kCols = 8;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
-    for (int k = 0; k < a.r.K; ++k) {
+    for (int k = warp; k < a.r.K; k += nw) {
         const long long* col = a.rpart + (size_t)k * a.nblk_q;
         long long v = 0;
-        for (int blk = t; blk < a.nblk_q; blk += blockDim.x) v += __ldcg(col + blk);
+        for (int b0 = lane; b0 < a.nblk_q; b0 += 32 * kCols) {
+            long long x[kCols];
+#pragma unroll
+            for (int u = 0; u < kCols; ++u) x[u] = b0 + 32 * u < a.nblk_q ? __ldcg(col + b0 + 32 * u) : 0;
+#pragma unroll
+            for (int u = 0; u < kCols; ++u) v += x[u];
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red64[warp * a.r.K + k] = v;
-    }
-    __syncthreads();
-    if (t < a.r.K) {
-        long long tot = 0;
-        for (int w = 0; w < nw; ++w) tot += red64[w * a.r.K + t];
-        const float v = (float)((double)tot * 2.3283064365386962890625e-10);
-        red[t] = v;
-        if (a.dd) a.dd[t] = v;
+        if (lane == 0) {
+            const float s = (float)((double)v * 2.3283064365386962890625e-10);
+            red[k] = s;
+            if (a.dd) a.dd[k] = s;
+        }
     }
     __syncthreads();
     if (t == 0 && a.dtheta) {

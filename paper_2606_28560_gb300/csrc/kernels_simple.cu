@@ -402,8 +402,7 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads) bwd_key_kernel(BwdArgs a) {
     grid_dependency_sync();
     __shared__ float red[kMaxRungs];
-    __shared__ long long red64[(kThreads / 32) * kMaxRungs];
-    if (blockIdx.x == 0 && a.want_dd) convert_rung_sums(a, red, red64);
+    if (blockIdx.x == 0 && a.want_dd) convert_rung_sums(a, red);
     const Shape s = a.s;
     const int c = threadIdx.x & 3;
     const int tiles = (s.T + kRowsPerBlock - 1) / kRowsPerBlock;
