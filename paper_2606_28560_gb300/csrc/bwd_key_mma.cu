@@ -204,7 +204,7 @@ bwd_key_mma_kernel(const __grid_constant__ RowMaps tmQ, const __grid_constant__ 
     // per warp: rung values of its slab columns; after a pass, its output rows
     __shared__ __align__(16) float rvals[kWarps][kMmaMaxRungs][16];
     __shared__ float wils[kWarps][32];                    // per warp: 1 / row sum of its band queries
-    __shared__ float red[kMmaMaxRungs];                   // block 0: dL/dd_k
+    __shared__ double red[kMmaMaxRungs];                   // block 0: dL/dd_k
     unsigned char* buf = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const unsigned sbase = smem_u32(buf);
 

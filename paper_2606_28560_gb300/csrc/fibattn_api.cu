@@ -166,7 +166,7 @@ ResLayout res_layout(int B, int H, int T, int W, int K) {
 }
 
 struct BwdLayout {
-    size_t qt, kt, P, DP, Delta, rpart, total;
+    size_t qt, kt, P, DP, rpart, total;
 };
 
 BwdLayout bwd_layout(int B, int H, int Hkv, int T, int W, int K, int dtype, bool own_kt) {
@@ -179,12 +179,11 @@ BwdLayout bwd_layout(int B, int H, int Hkv, int T, int W, int K, int dtype, bool
     if (own_kt) off += align256((size_t)B * Hkv * T * kHeadDim * es);   // else the caller's rotated_k
     L.P = off; off += align256((size_t)B * H * T * S * 4);
     L.DP = off; off += align256((size_t)B * H * T * S * 4);
-    L.Delta = off; off += align256((size_t)B * H * T * 4);
     L.rpart = off;                                  // fixed-point rung partials, one per query block
     Shape s;
     std::memset(&s, 0, sizeof(s));
     s.B = B; s.H = H; s.Hkv = Hkv; s.T = T; s.W = W; s.G = H / Hkv;
-    off += align256((size_t)kMaxRungs * 8 * std::max(bwd_simple_blocks(s), bwd_mma_blocks(s)));
+    off += align256((size_t)K * 8 * std::max(bwd_gather_blocks(s), bwd_mma_blocks(s)));
     L.total = off;
     return L;
 }
@@ -472,7 +471,7 @@ int fibattn_fwd(const void* q, const void* k, const void* v, void* out, float* l
         e = launch_fwd_mma(a, ML, st);
     } else {
         ProfScope p("fwd", st);
-        e = launch_fwd_simple(a, bf16, st);
+        e = launch_fwd_gather(a, bf16, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "forward launch");
     return FIBATTN_OK;
@@ -513,10 +512,8 @@ int fibattn_bwd(const void* q, const void* k, const void* v, const void* out, co
     a.dtheta = dtheta; a.dd = dd;
     a.want_dd = (dtheta || dd) ? 1 : 0;
     a.qt = ws + L.qt; a.kt = o.rotated_k ? o.rotated_k : ws + L.kt;
-    a.P = reinterpret_cast<float*>(ws + L.P); a.DP = reinterpret_cast<float*>(ws + L.DP);
-    a.Delta = reinterpret_cast<float*>(ws + L.Delta);
     a.rpart = reinterpret_cast<long long*>(ws + L.rpart);
-    a.nblk_q = bwd_simple_blocks(a.s);
+    a.nblk_q = bwd_gather_blocks(a.s);
     a.S = W + 1 + K;
     a.alpha = alpha;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
@@ -526,7 +523,7 @@ int fibattn_bwd(const void* q, const void* k, const void* v, const void* out, co
     const bool mma_ok = bf16 && out && (o.bwd_kernel == 0 || o.bwd_kernel == 2) &&
                         build_mma_layout(a.s, a.r, o.rope_base, smem_limit, &ML, 3 * kTileRows) &&
                         build_key_layout(a.s, a.r, o.rope_base, 227 * 1024 - bwd_key_mma_static_smem(), &KL);
-    a.Ps = reinterpret_cast<float*>(ws + L.P);      // slot-major p and dS of the tensor-core passes
+    a.Ps = reinterpret_cast<float*>(ws + L.P);      // slot-major p and dS
     a.DSs = reinterpret_cast<float*>(ws + L.DP);
     if (o.bwd_kernel == 2 && !mma_ok)
         return fail(FIBATTN_ERR_UNSUPPORTED, "tensor-core backward needs bf16, out, W <= 16, K <= 16 and a staged row "
@@ -546,11 +543,6 @@ int fibattn_bwd(const void* q, const void* k, const void* v, const void* out, co
     if ((rc = bind_context())) return rc;
     if ((rc = status_word(&a.status))) return rc;
     if (B > 0) {
-        if (!mma_ok) {
-            ProfScope p("rope_q", st);
-            e = launch_rope_rows(q, a.qt, (long long)B * H * T, T, a.rope, bf16, st, a.status);
-            if (e != cudaSuccess) return cuda_fail(e, "rope prologue (q) launch");
-        }
         if (!o.rotated_k) {                      // else the rotated keys come from the forward
             ProfScope p("rope_k", st);
             e = launch_rope_rows(k, a.kt, (long long)B * o.Hkv * T, T, a.rope, bf16, st, a.status);
@@ -561,7 +553,7 @@ int fibattn_bwd(const void* q, const void* k, const void* v, const void* out, co
             e = launch_bwd_query_mma(a, ML, st);
         } else {
             ProfScope p("bwd_query", st);
-            e = launch_bwd_query(a, bf16, st);
+            e = launch_bwd_query_gather(a, bf16, st);
         }
         if (e != cudaSuccess) return cuda_fail(e, "backward query-pass launch");
         if (mma_ok) {
@@ -569,7 +561,7 @@ int fibattn_bwd(const void* q, const void* k, const void* v, const void* out, co
             e = launch_bwd_key_mma(a, KL, st);
         } else {
             ProfScope p("bwd_key", st);
-            e = launch_bwd_key(a, bf16, st);
+            e = launch_bwd_key_gather(a, bf16, st);
         }
         if (e != cudaSuccess) return cuda_fail(e, "backward key-pass launch");
     }

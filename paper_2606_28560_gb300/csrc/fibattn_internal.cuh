@@ -107,14 +107,11 @@ struct BwdArgs {
     int want_dd;              // compute dL/dd_k (dtheta or dd requested)
     float* dd;                // device [K] or nullptr
     // workspace views
-    void* qt;                 // rotated q [B,H,T,D] (bf16 from the tensor-core query pass, fp16 from the prologue)
+    void* qt;                 // rotated q [B,H,T,D] from the query pass (tensor-core: bf16; row-gather: fp16, or fp32 for fp32 I/O)
     void* kt;                 // rotated k [B,Hkv,T,D]
-    float* P;                 // softmax probabilities [B,H,T,S]
-    float* DP;                // dL/dp = dO . val per slot [B,H,T,S]
-    float* Delta;             // sum_slots p dL/dp per query [B,H,T]
-    float* Ps;                // tensor-core path, slot-major [B,H,S,T]: p      (P region)
-    float* DSs;               //                                      dS = p (dp - Delta)  (DP region)
-    long long* rpart;         // per query-pass block dL/dd_k partials, 2^-32 fixed point [kMaxRungs][nblk_q]
+    float* Ps;                // slot-major [B,H,S,T]: p
+    float* DSs;               //                       dS = p (dp - Delta)
+    long long* rpart;         // per query-pass block dL/dd_k partials, 2^-32 fixed point [K][nblk_q]
     const float* res_il;      // forward residual 1 / (row sum) [B,H,T] (p = Ps[slot] * res_il)
     const float* res_sd;      // forward residual far-minus-floor rung scores [B,H,K,T], or nullptr;
                               // when the forward residuals are used, Ps and qt point into them
@@ -138,104 +135,32 @@ __device__ __forceinline__ void rope_cs(const RopeParams& rp, int m, int pos, fl
     __sincosf(ang, &s, &c);
 }
 
-// ------------------------------------------------------------- element IO --
+// cos/sin of the same angle to fp32 rounding, for fp32 I/O (rope_cs is off by
+// up to 4e-7, the largest error of that path: dL/dd_k 3.3e-7 off 64 bits with
+// it, 2e-7 without).  The phase is reduced to an eighth of a turn either side
+// of a multiple of a quarter turn as an integer, exactly; the Taylor
+// polynomials of sine and cosine to the 9th and 10th power do the rest (the
+// first terms left out are below 2e-9).
+__device__ __forceinline__ void rope_cs_exact(const RopeParams& rp, int m, int pos, float& c, float& s) {
+    const unsigned ph = (unsigned)(((unsigned long long)(unsigned)pos * rp.F[m]) >> 32);
+    const unsigned quarter = (ph + 0x20000000u) >> 30;            // nearest multiple of a quarter turn
+    const float x = (float)(int)(ph - (quarter << 30)) * 1.4629180792671596e-09f;   // 2 pi / 2^32
+    const float y = x * x;
+    const float sn = fmaf(x * y, fmaf(y, fmaf(y, fmaf(y, 1.f / 362880.f, -1.f / 5040.f), 1.f / 120.f), -1.f / 6.f), x);
+    const float cn = fmaf(y, fmaf(y, fmaf(y, fmaf(y, fmaf(y, -1.f / 3628800.f, 1.f / 40320.f), -1.f / 720.f), 1.f / 24.f),
+                                  -0.5f), 1.f);
+    const bool swap = quarter & 1u;
+    c = swap ? sn : cn;
+    s = swap ? cn : sn;
+    if (quarter == 1u || quarter == 2u) c = -c;
+    if (quarter >= 2u) s = -s;
+}
 
-__device__ __forceinline__ float to_f(float x) { return x; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
-
-template <typename T> struct Vec8;   // 8 consecutive elements
-
-template <> struct Vec8<float> {
-    static __device__ __forceinline__ void load(const float* p, float* x) {
-        float4 a = *reinterpret_cast<const float4*>(p);
-        float4 b = *reinterpret_cast<const float4*>(p + 4);
-        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-    }
-    static __device__ __forceinline__ void store(float* p, const float* x) {
-        *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
-        *reinterpret_cast<float4*>(p + 4) = make_float4(x[4], x[5], x[6], x[7]);
-    }
-};
-
-template <> struct Vec8<__nv_bfloat16> {
-    static __device__ __forceinline__ void load(const __nv_bfloat16* p, float* x) {
-        uint4 u = *reinterpret_cast<const uint4*>(p);
-        unsigned w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            x[2 * i] = __uint_as_float(w[i] << 16);
-            x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-        }
-    }
-    static __device__ __forceinline__ void store(__nv_bfloat16* p, const float* x) {
-        uint4 u;
-        unsigned w[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * i], x[2 * i + 1]);
-            w[i] = *reinterpret_cast<unsigned*>(&h);
-        }
-        u.x = w[0]; u.y = w[1]; u.z = w[2]; u.w = w[3];
-        *reinterpret_cast<uint4*>(p) = u;
-    }
-};
-
-// fp16 holds the RoPE-rotated q/k rows of the bf16 path: 10 mantissa bits
-// against bf16's 7 keep the score error well inside the bf16 tolerance.
-template <> struct Vec8<__half> {
-    static __device__ __forceinline__ void load(const __half* p, float* x) {
-        uint4 u = *reinterpret_cast<const uint4*>(p);
-        unsigned w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float2 f = __half22float2(*reinterpret_cast<__half2*>(&w[i]));
-            x[2 * i] = f.x;
-            x[2 * i + 1] = f.y;
-        }
-    }
-    static __device__ __forceinline__ void store(__half* p, const float* x) {
-        uint4 u;
-        unsigned w[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            __half2 h = __floats2half2_rn(x[2 * i], x[2 * i + 1]);
-            w[i] = *reinterpret_cast<unsigned*>(&h);
-        }
-        u.x = w[0]; u.y = w[1]; u.z = w[2]; u.w = w[3];
-        *reinterpret_cast<uint4*>(p) = u;
-    }
-};
-
-// Storage type of rotated rows: fp32 for fp32 I/O, fp16 for bf16 I/O.
+// Storage type of rotated rows: fp32 for fp32 I/O, fp16 for bf16 I/O (10
+// mantissa bits against bf16's 7 keep the score error well inside the bf16
+// tolerance).
 template <typename T> struct RotOf { using type = float; };
 template <> struct RotOf<__nv_bfloat16> { using type = __half; };
-
-// A lane of a 4-lane group owns RoPE pairs [8c, 8c+8): head dims 8c..8c+7
-// (x[0..7]) and 32+8c..32+8c+7 (x[8..15]), so a rotation stays in the lane.
-template <typename T>
-__device__ __forceinline__ void load_chunk(const T* row, int c, float* x) {
-    Vec8<T>::load(row + 8 * c, x);
-    Vec8<T>::load(row + kHalf + 8 * c, x + 8);
-}
-template <typename T>
-__device__ __forceinline__ void store_chunk(T* row, int c, const float* x) {
-    Vec8<T>::store(row + 8 * c, x);
-    Vec8<T>::store(row + kHalf + 8 * c, x + 8);
-}
-
-// x <- R(pos) x (inverse = false) or R(pos)^T x (inverse = true) for the 8
-// pairs owned by lane c.
-__device__ __forceinline__ void rope_chunk(const RopeParams& rp, int pos, int c, float* x, bool inverse) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        float cs, sn;
-        rope_cs(rp, 8 * c + u, pos, cs, sn);
-        if (inverse) sn = -sn;
-        float a = x[u], b = x[8 + u];
-        x[u] = a * cs - b * sn;
-        x[8 + u] = b * cs + a * sn;
-    }
-}
 
 // ------------------------------------------------- rung-gradient reduction --
 
@@ -252,14 +177,14 @@ __device__ __forceinline__ void write_rung_partials(const BwdArgs& a, float part
 }
 
 // Called by every thread of one block of the key pass (blockDim a multiple of
-// 32).  red: shared scratch of at least K floats.  A warp sums whole rungs,
+// 32).  red: shared scratch of at least K doubles.  A warp sums whole rungs,
 // kCols columns a lane in flight at a time.  Bound by load latency: one thread
 // block adds K x (query-pass blocks) words while others may already be done.
 // Rung after rung over all threads (a latency and a warp sum
 // each) it was the end of the whole backward on small grids: key pass at B1
 // H8 T1000 17.7 -> 12.5 us, at B4 22.6 -> 18.4 us, at B16 H8 Hkv2 T1024 (its
 // blocks fit one wave) 47.3 -> 41.7 us; unchanged where several waves hide it.
-__device__ __forceinline__ void convert_rung_sums(const BwdArgs& a, float* red) {
+__device__ __forceinline__ void convert_rung_sums(const BwdArgs& a, double* red) {
     constexpr int kCols = 8;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
     for (int k = warp; k < a.r.K; k += nw) {
@@ -275,16 +200,15 @@ __device__ __forceinline__ void convert_rung_sums(const BwdArgs& a, float* red) 
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) {
-            const float s = (float)((double)v * 2.3283064365386962890625e-10);
-            red[k] = s;
-            if (a.dd) a.dd[k] = s;
+            red[k] = (double)v * 2.3283064365386962890625e-10;
+            if (a.dd) a.dd[k] = (float)red[k];
         }
     }
     __syncthreads();
     if (t == 0 && a.dtheta) {
-        float da = 0.f;
-        for (int k = 0; k < a.r.K; ++k) da += a.r.f[k] * red[k];
-        *a.dtheta = da * (a.alpha - 0.5f) * (1.5f - a.alpha);
+        double da = 0.0;                          // (the terms cancel: an fp32 sum would add error of its own)
+        for (int k = 0; k < a.r.K; ++k) da += (double)a.r.f[k] * red[k];
+        *a.dtheta = (float)(da * ((double)a.alpha - 0.5) * (1.5 - (double)a.alpha));
     }
 }
 
@@ -331,10 +255,11 @@ cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t 
 
 cudaError_t launch_rope_rows(const void* src, void* dst, long long rows, int T, const RopeParams& rp,
                              bool bf16, cudaStream_t st, unsigned* status);
-cudaError_t launch_fwd_simple(const FwdArgs& a, bool bf16, cudaStream_t st);
-cudaError_t launch_bwd_query(const BwdArgs& a, bool bf16, cudaStream_t st);
-cudaError_t launch_bwd_key(const BwdArgs& a, bool bf16, cudaStream_t st);
-int bwd_simple_blocks(const Shape& s);
+// The row-gather passes (gather.cu).
+cudaError_t launch_fwd_gather(const FwdArgs& a, bool bf16, cudaStream_t st);
+cudaError_t launch_bwd_query_gather(const BwdArgs& a, bool bf16, cudaStream_t st);
+cudaError_t launch_bwd_key_gather(const BwdArgs& a, bool bf16, cudaStream_t st);
+int bwd_gather_blocks(const Shape& s);            // query-pass blocks: columns of BwdArgs::rpart
 
 // Records a message for fibattn_last_error() and returns `code`.
 int set_error(int code, const char* msg);
