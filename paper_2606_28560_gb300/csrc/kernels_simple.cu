@@ -18,11 +18,14 @@ namespace {
 // position, chunk c): dims 8c..8c+7 and their RoPE partners 32+8c..32+8c+7;
 // a warp covers the tile's 8 positions x 4 chunks of one head (1 KB
 // contiguous), and a thread issues the loads of all its items (TH / 8)
-// before any arithmetic.
+// before any arithmetic.  Four blocks an SM (64 registers; 70 allowed three):
+// the 512 tiles of B16 H8 T1024 are then all resident at once, where the last
+// 56 had to wait for a slot (forward with the rotation 38.7 -> 38.3 us, at B4
+// T4096 41.2 -> 40.6 us).
 constexpr int kRopePos = 8;
 constexpr int kRopeTabStride = 34;            // floats per position (32 + pad: conflict-free float2 reads)
 template <int TH>
-__global__ void __launch_bounds__(256) rope_rows_bf16_kernel(const __nv_bfloat16* __restrict__ src,
+__global__ void __launch_bounds__(256, 4) rope_rows_bf16_kernel(const __nv_bfloat16* __restrict__ src,
                                                              __half* __restrict__ dst, int heads, int T_,
                                                              RopeParams rp, unsigned* status) {
     constexpr int kItems = TH / 8;                // per thread (256 threads)
@@ -142,7 +145,9 @@ cudaError_t launch_rope_rows(const void* src, void* dst, long long rows, int T, 
         // they free up, which balances the load better than a grid-stride
         // loop); tiles of 32 heads while they still give two blocks per SM,
         // else of 16 (B16 H8 T1024: 2.296 -> 2.281 ms per 16-layer step;
-        // with two kv heads, 512 tiles of 16 heads beat 128 of 32)
+        // with two kv heads, 512 tiles of 16 heads beat 128 of 32), and never
+        // of 32 where 16 rows are all there are (B2 H8 T16384: rotation 17.9
+        // -> 16.2 us)
         static int sms = 0;
         if (sms == 0) {
             int dev = 0;
@@ -153,7 +158,7 @@ cudaError_t launch_rope_rows(const void* src, void* dst, long long rows, int T, 
         const long long t32 = tp * ((heads + 31) / 32), t16 = tp * ((heads + 15) / 16);
         const __nv_bfloat16* s16 = reinterpret_cast<const __nv_bfloat16*>(src);
         __half* d16 = reinterpret_cast<__half*>(dst);
-        if (t32 >= 2LL * sms)
+        if (t32 >= 2LL * sms && heads > 16)
             return launch_kernel(rope_rows_bf16_kernel<32>, dim3((unsigned)std::min(t32, 0x7fffffffLL)), dim3(256),
                                  0, st, s16, d16, heads, T, rp, status);
         return launch_kernel(rope_rows_bf16_kernel<16>, dim3((unsigned)std::min(t16, 0x7fffffffLL)), dim3(256), 0,
