@@ -24,7 +24,7 @@ from . import binding as B
 def alpha_of_theta(theta: float) -> float:
     """alpha = 0.5 + sigmoid(theta) (Section 2, "The per-layer scalar"), as the
     library computes it (fibattn_alpha_schedule, learned kind)."""
-    return float(B.alpha_schedule("learned", 1, theta=[float(theta)])[0])
+    return B.alpha_of_theta(float(theta))
 
 
 class FibAttentionFunction(torch.autograd.Function):
@@ -36,22 +36,10 @@ class FibAttentionFunction(torch.autograd.Function):
     def forward(ctx, q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha=None):
         if alpha is None:
             alpha = alpha_of_theta(float(theta))
-        rk = B.rotated_k_like(k)
-        kw = dict(rope_base=rope_base, scale=scale, dedup=dedup, rotated_k=rk)
-        res = None
-        if q.dtype == torch.bfloat16:
-            # the tensor-core forward also keeps p, the rung score differences and
-            # the rotated queries, so the backward does not recompute the scores
-            res = B.residuals_like(q, W, len(offsets))
-            try:
-                out, lse = B.fwd(q, k, v, alpha, offsets, W, residuals=res, **kw)
-            except B.FibattnError as e:
-                if e.status != B.FIBATTN_ERR_UNSUPPORTED:
-                    raise
-                res = None
-        if res is None:
-            out, lse = B.fwd(q, k, v, alpha, offsets, W, **kw)
-            res = torch.empty(0, dtype=torch.uint8, device=q.device)
+        # for bf16 I/O the tensor-core forward also keeps p, the rung score
+        # differences and the rotated queries, so the backward does not recompute
+        # the scores
+        out, lse, rk, res = B.fwd_keep(q, k, v, alpha, offsets, W, rope_base=rope_base, scale=scale, dedup=dedup)
         ctx.save_for_backward(q, k, v, out, lse, rk, res)
         ctx.args = (alpha, offsets, W, rope_base, scale, dedup, theta.dtype, theta.device)
         return out
@@ -62,9 +50,26 @@ class FibAttentionFunction(torch.autograd.Function):
         alpha, offsets, W, rope_base, scale, dedup, tdtype, tdev = ctx.args
         dq, dk, dv, dth, _ = B.bwd(q, k, v, lse, dout.contiguous(), alpha, offsets, W, out=out,
                                    rope_base=rope_base, scale=scale, dedup=dedup, rotated_k=rk,
-                                   residuals=res if res.numel() else None)
-        dtheta = dth.reshape(()).to(device=tdev, dtype=tdtype)
+                                   residuals=res)
+        dtheta = dth.reshape(())
+        if dtheta.device != tdev or dtheta.dtype != tdtype:
+            dtheta = dtheta.to(device=tdev, dtype=tdtype)
         return dq, dk, dv, dtheta, None, None, None, None, None, None
+
+
+def _attend(q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha):
+    """FibAttentionFunction, or the forward alone where no gradient is asked
+    for: it then keeps nothing for a backward (the residuals add half again to
+    the forward's traffic) and autograd takes no part.  A call inside a
+    function transform or forward-mode differentiation goes to autograd, which
+    refuses it."""
+    alpha = None if alpha is None else float(alpha)
+    if (torch.is_grad_enabled() and (q.requires_grad or k.requires_grad or v.requires_grad or theta.requires_grad)) \
+            or torch._C._are_functorch_transforms_active() or torch.autograd.forward_ad._current_level >= 0:
+        return FibAttentionFunction.apply(q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha)
+    if alpha is None:
+        alpha = alpha_of_theta(float(theta))
+    return B.fwd(q, k, v, alpha, offsets, W, rope_base=rope_base, scale=scale, dedup=dedup)[0]
 
 
 def fib_attention(q, k, v, theta, offsets=None, W: int = 8, *, rope_base: float = 1e4, scale=None,
@@ -78,8 +83,7 @@ def fib_attention(q, k, v, theta, offsets=None, W: int = 8, *, rope_base: float 
         offsets = B.base("fib", 15)
     if not torch.is_tensor(theta):
         theta = torch.tensor(float(theta))
-    return FibAttentionFunction.apply(q, k, v, theta, offsets, W, rope_base, scale, dedup,
-                                      None if alpha is None else float(alpha))
+    return _attend(q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha)
 
 
 class FibAttention(torch.nn.Module):
@@ -104,8 +108,7 @@ class FibAttention(torch.nn.Module):
     def forward(self, q, k, v, alpha=None):
         """``alpha``: the host value of 0.5 + sigmoid(theta), when the caller
         has read it (skips the per-call read of a theta on the GPU)."""
-        return FibAttentionFunction.apply(q, k, v, self.theta, self.offsets, self.W, self.rope_base, self.scale,
-                                          self.dedup, None if alpha is None else float(alpha))
+        return _attend(q, k, v, self.theta, self.offsets, self.W, self.rope_base, self.scale, self.dedup, alpha)
 
 
 def theta_of_alpha(alpha: float) -> float:
@@ -122,7 +125,10 @@ def attention_stack(x: torch.Tensor, layers) -> torch.Tensor:
     if not layers:
         return x
     dev = layers[0].theta.device
-    thetas = torch.stack([layer.theta.detach().to(device=dev, dtype=torch.float32) for layer in layers]).tolist()
+    if all(layer.theta.device.type == "cpu" for layer in layers):
+        thetas = [layer.theta.item() for layer in layers]
+    else:
+        thetas = torch.stack([layer.theta.detach().to(device=dev, dtype=torch.float32) for layer in layers]).tolist()
     alphas = B.alpha_schedule("learned", len(layers), theta=thetas)
     for layer, a in zip(layers, alphas):
         x = layer(x, x, x, alpha=float(a))

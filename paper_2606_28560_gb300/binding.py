@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C ABI in ``include/fibattn.h``.
+"""Thin binding of the C ABI in ``include/fibattn.h``: ctypes for the host-side
+calls, and ``csrc/marshal.cpp`` for the two compute calls.
 
 Argument marshalling only: tensors are passed as raw device pointers with the
 caller's current CUDA stream; every step of the computation runs in the CUDA
@@ -9,6 +10,8 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import importlib.machinery
+import importlib.util
 import os
 import threading
 
@@ -85,6 +88,27 @@ def lib():
     return _lib
 
 
+_marshal_module = None
+
+
+def _marshal():
+    """The native marshalling module (built with the library)."""
+    global _marshal_module
+    if _marshal_module is None:
+        lib()
+        with _lock:
+            if _marshal_module is None:
+                path = _build.MARSHAL
+                if not os.path.exists(path):
+                    raise RuntimeError(f"native binding not built ({path} missing); run __graft_entry__.build()")
+                loader = importlib.machinery.ExtensionFileLoader("fibattn_marshal", path)
+                spec = importlib.util.spec_from_file_location("fibattn_marshal", path, loader=loader)
+                m = importlib.util.module_from_spec(spec)
+                loader.exec_module(m)
+                _marshal_module = m
+    return _marshal_module
+
+
 def _check(rc: int):
     if rc != 0:
         raise FibattnError(rc, lib().fibattn_last_error().decode(errors="replace"))
@@ -150,35 +174,10 @@ def residual_views(res: torch.Tensor, B, H, T, W, K):
     return qt, P, sd, il
 
 
-def _check_residuals(res, q, W, K):
-    if res is None:
-        return
-    B, H, T, D = q.shape
-    if not (res.is_cuda and res.is_contiguous() and res.numel() * res.element_size() >=
-            residual_bytes(B, H, T, W, K, q.dtype, D)):
-        raise ValueError("residuals must be a contiguous CUDA buffer of residual_bytes(...) bytes")
-
-
 def rotated_k_like(k: torch.Tensor) -> torch.Tensor:
     """A buffer for the rotated keys (``rotated_k=``): fp16 for bf16 k, fp32 for fp32 k."""
     return torch.empty(k.shape, dtype=torch.float16 if k.dtype == torch.bfloat16 else torch.float32,
                        device=k.device)
-
-
-def _check_rotated(rk, k):
-    if rk is None:
-        return
-    want = torch.float16 if k.dtype == torch.bfloat16 else torch.float32
-    if not (rk.is_cuda and rk.is_contiguous() and rk.dtype == want and rk.shape == k.shape):
-        raise ValueError(f"rotated_k must be a contiguous CUDA {want} tensor of k's shape")
-
-
-def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return FIBATTN_F32
-    if t.dtype == torch.bfloat16:
-        return FIBATTN_BF16
-    raise TypeError(f"unsupported dtype {t.dtype}: fp32 or bf16")
 
 
 def _stream_ptr(stream) -> int:
@@ -193,6 +192,11 @@ def _offsets(offsets) -> np.ndarray:
 
 
 # ------------------------------------------------------------- host prep ----
+
+def alpha_of_theta(theta: float) -> float:
+    """0.5 + sigmoid(theta) (fibattn_alpha_schedule, learned kind)."""
+    return (_marshal_module or _marshal()).alpha_of_theta(theta)
+
 
 def base(kind: str, K: int) -> np.ndarray:
     f = np.zeros(K, dtype=np.float32)
@@ -288,28 +292,23 @@ def fwd(q, k, v, alpha: float, offsets, W: int, *, rope_base=1e4, scale=None, de
     optional buffer (``residuals_like(q, W, K)``) that receives the rotated
     queries, p of every slot and the rung score differences for a later
     ``bwd(..., residuals=...)`` (tensor-core forward only).  Returns (out, lse)."""
-    B, H, T, D = q.shape
-    Hkv = k.shape[1]
-    f = _offsets(offsets)
-    _check_rotated(rotated_k, k)
-    _check_residuals(residuals, q, W, len(f))
-    o = _opts(rope_base, scale, Hkv, dedup, kernel, rotated_k=rotated_k, residuals=residuals,
-              round_offsets=round_offsets)
-    code = _dtype_code(q)
-    for t in (q, k, v):
-        if not (t.is_cuda and t.is_contiguous() and t.dtype == q.dtype):
-            raise ValueError("q, k, v must be contiguous CUDA tensors of one dtype")
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((B, H, T), dtype=torch.float32, device=q.device)
-    if workspace is None:                        # (a given workspace's size is checked by the library)
-        need = int(lib().fibattn_fwd_workspace_bytes(B, H, T, D, W, len(f), code, ctypes.byref(o)))
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device)
-    _check(lib().fibattn_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), lse.data_ptr(),
-                             B, H, T, D, int(W), float(alpha), f.ctypes.data, len(f), code, ctypes.byref(o),
-                             workspace.data_ptr(), workspace.numel(), _stream_ptr(stream)))
-    return out, lse
+    r = (_marshal_module or _marshal()).fwd(
+        q, k, v, _offsets(offsets), int(W), alpha, rope_base, scale or 0.0, dedup, round_offsets, FWD_KERNELS[kernel], out,
+        lse, workspace, rotated_k, residuals, None if stream is None else stream.cuda_stream)
+    if r.__class__ is int:
+        _check(r)
+    return r
+
+
+def fwd_keep(q, k, v, alpha: float, offsets, W: int, *, rope_base=1e4, scale=None, dedup=True):
+    """The forward pass of a training step, on the current stream: (out, lse,
+    rotated_k, residuals) with the buffers a later ``bwd`` takes (residuals
+    None where the tensor-core forward does not apply)."""
+    r = (_marshal_module or _marshal()).fwd_keep(q, k, v, _offsets(offsets), int(W), alpha, rope_base, scale or 0.0,
+                                                 dedup, False)
+    if r.__class__ is int:
+        _check(r)
+    return r
 
 
 def bwd(q, k, v, lse, dout, alpha: float, offsets, W: int, *, out=None, rope_base=1e4, scale=None, dedup=True,
@@ -324,37 +323,13 @@ def bwd(q, k, v, lse, dout, alpha: float, offsets, W: int, *, out=None, rope_bas
     dL/dtheta and dL/dd_k (a fixed schedule; required with ``round_offsets``).
     Returns (dq, dk, dv, dtheta [1], dd [K]) on the device (dtheta, dd None
     without rung_grads)."""
-    B, H, T, D = q.shape
-    Hkv = k.shape[1]
-    f = _offsets(offsets)
-    K = len(f)
-    _check_rotated(rotated_k, k)
-    _check_residuals(residuals, q, W, K)
-    o = _opts(rope_base, scale, Hkv, dedup, bwd_kernel=kernel, rotated_k=rotated_k, residuals=residuals,
-              round_offsets=round_offsets)
-    code = _dtype_code(q)
-    for t in (q, k, v, dout) + ((out,) if out is not None else ()):
-        if not (t.is_cuda and t.is_contiguous() and t.dtype == q.dtype):
-            raise ValueError("q, k, v, dout, out must be contiguous CUDA tensors of one dtype")
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(k) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    if rung_grads:
-        dtheta = torch.empty(4, dtype=torch.float32, device=q.device) if dtheta is None else dtheta
-        dd = torch.empty(max(K, 1), dtype=torch.float32, device=q.device) if dd is None else dd
-    if workspace is None:                        # (a given workspace's size is checked by the library)
-        need = int(lib().fibattn_bwd_workspace_bytes(B, H, T, D, W, K, code, ctypes.byref(o)))
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device)
-    _check(lib().fibattn_bwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr() if out is not None else None,
-                             lse.data_ptr(), dout.data_ptr(),
-                             dq.data_ptr(), dk.data_ptr(), dv.data_ptr(),
-                             dtheta.data_ptr() if dtheta is not None else None,
-                             dd.data_ptr() if dd is not None else None,
-                             B, H, T, D, int(W), float(alpha), f.ctypes.data, K, code, ctypes.byref(o),
-                             workspace.data_ptr(), workspace.numel(), _stream_ptr(stream)))
-    if dtheta is None and dd is None:
-        return dq, dk, dv, None, None
-    return dq, dk, dv, (dtheta[:1] if dtheta is not None else None), (dd[:K] if dd is not None else None)
+    r = (_marshal_module or _marshal()).bwd(
+        q, k, v, _offsets(offsets), int(W), alpha, rope_base, scale or 0.0, dedup, round_offsets, BWD_KERNELS[kernel], out,
+        lse, workspace, rotated_k, residuals, None if stream is None else stream.cuda_stream, dout, dq, dk, dv, dtheta,
+        dd, rung_grads)
+    if r.__class__ is int:
+        _check(r)
+    return r
 
 
 # ---------------------------------------------------------- device status ----

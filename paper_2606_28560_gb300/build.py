@@ -1,8 +1,9 @@
 """Build the CUDA library in-tree for sm_103a (GB300) with nvcc.
 
 Each ``csrc/*.cu`` translation unit is compiled in parallel, then linked into
-``_build/libfibattn.so`` against the shared CUDA runtime.  Rebuilds only when
-a source or header is newer than the library.
+``_build/libfibattn.so`` against the shared CUDA runtime; ``csrc/marshal.cpp``
+is compiled with g++ against PyTorch's headers into ``_build/fibattn_marshal.so``.
+Rebuilds only when a source or header is newer than the libraries.
 """
 from __future__ import annotations
 
@@ -10,6 +11,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -17,6 +19,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libfibattn.so")
+MARSHAL = os.path.join(BUILD, "fibattn_marshal.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
               "-Xptxas", "-warn-spills"]
@@ -38,13 +41,13 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    return _sources() + [os.path.join(CSRC, "marshal.cpp")] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(MARSHAL)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
@@ -65,8 +68,24 @@ def build(force: bool = False, verbose: bool = False) -> str:
             print(r.stderr)
         return obj
 
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    tlib = os.path.join(tdir, "lib")
+    marshal_obj = os.path.join(BUILD, "marshal.cpp.o")
+
+    def compile_marshal(_):
+        inc = [os.path.join(tdir, "include"), os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include")]
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               *[f"-I{d}" for d in inc], "-c", os.path.join(CSRC, "marshal.cpp"), "-o", marshal_obj]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"g++ failed on marshal.cpp:\n{r.stderr}")
+
     with ThreadPoolExecutor(max_workers=max(1, min(8, os.cpu_count() or 1))) as ex:
+        marshal = ex.submit(compile_marshal, None)
         objs = list(ex.map(compile_one, _sources()))
+        marshal.result()
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc, *ARCH, "-shared", "-cudart", "shared", "-o", tmp, *objs,
            "-Xlinker", f"-rpath={cuda_lib}"]
@@ -74,6 +93,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stderr}")
     os.replace(tmp, LIB)
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    cmd = ["g++", "-shared", "-o", tmp, marshal_obj, f"-L{BUILD}", "-lfibattn", f"-L{tlib}", "-lc10", "-lc10_cuda",
+           "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{tlib}", f"-Wl,-rpath,{cuda_lib}"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"link of marshal failed:\n{r.stderr}")
+    os.replace(tmp, MARSHAL)
     return LIB
 
 

@@ -33,6 +33,7 @@
 // output rows (and the rotated query rows it keeps) through a 1 KB stage per
 // warp, as 16-byte pieces of runs of consecutive rows.
 #include <cmath>
+#include <cstring>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -699,12 +700,19 @@ void active_list(const RungParams& r, MmaLayout* L) {
     L->win_iv = interval_of(*L, L->win_smem);
 }
 
+// (a thread keeps the table of the last base, as prep_rope does)
 void rope_steps(double rope_base, MmaLayout* L) {
-    for (int m = 0; m < kHalf; ++m) {
-        const double theta = std::pow(rope_base, -2.0 * m / (double)kHeadDim);
-        L->rope_c8[m] = (float)std::cos(8.0 * theta);
-        L->rope_s8[m] = (float)std::sin(8.0 * theta);
+    static thread_local struct { double base = 0.0; float c8[kHalf], s8[kHalf]; } last;
+    if (last.base != rope_base) {
+        for (int m = 0; m < kHalf; ++m) {
+            const double theta = std::pow(rope_base, -2.0 * m / (double)kHeadDim);
+            last.c8[m] = (float)std::cos(8.0 * theta);
+            last.s8[m] = (float)std::sin(8.0 * theta);
+        }
+        last.base = rope_base;
     }
+    std::memcpy(L->rope_c8, last.c8, sizeof(last.c8));
+    std::memcpy(L->rope_s8, last.s8, sizeof(last.s8));
 }
 
 }  // namespace

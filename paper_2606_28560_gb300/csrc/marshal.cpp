@@ -1,0 +1,259 @@
+// marshal.cpp -- the two compute calls of include/fibattn.h for PyTorch
+// tensors: checks, output allocation and the call, natively.  binding.py holds
+// the signatures; nothing of the computation is here.  A forward call of
+// B1 H8 Hkv2 T64 took 36-43 us of host time interpreted (its kernels 10), and
+// takes 12-13 us here (GB300, Grace host).
+#include <Python.h>
+
+#include <ATen/core/Tensor.h>
+#include <ATen/ops/empty.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "../../include/fibattn.h"
+
+namespace {
+
+using at::Tensor;
+
+[[noreturn]] void value_error(const char* msg) {
+    PyErr_SetString(PyExc_ValueError, msg);
+    throw python_error();
+}
+
+const Tensor& tensor(PyObject* o, const char* name) {
+    if (!THPVariable_Check(o)) {
+        PyErr_Format(PyExc_TypeError, "%s must be a tensor, not %s", name, Py_TYPE(o)->tp_name);
+        throw python_error();
+    }
+    return THPVariable_Unpack(o);
+}
+// None reads as an undefined tensor.
+Tensor optional(PyObject* o, const char* name) { return o == Py_None ? Tensor() : tensor(o, name); }
+
+long as_int(PyObject* o) {
+    const long v = PyLong_AsLong(o);
+    if (v == -1 && PyErr_Occurred()) throw python_error();
+    return v;
+}
+double as_float(PyObject* o) {
+    const double v = PyFloat_AsDouble(o);
+    if (v == -1.0 && PyErr_Occurred()) throw python_error();
+    return v;
+}
+
+// The base sequence: a C-contiguous float32 array (binding.py makes it one).
+struct Offsets {
+    Py_buffer b;
+    const float* f;
+    int K;
+    explicit Offsets(PyObject* o) {
+        if (PyObject_GetBuffer(o, &b, PyBUF_ND | PyBUF_C_CONTIGUOUS) != 0) throw python_error();
+        f = static_cast<const float*>(b.buf);
+        K = b.ndim > 0 ? (int)b.shape[0] : -1;    // (refused by the library, as a scalar was by len())
+    }
+    ~Offsets() { PyBuffer_Release(&b); }
+};
+
+void* ptr(const Tensor& t) { return t.defined() ? t.data_ptr() : nullptr; }
+
+// Sizes, options and the checks both calls make.
+struct Call {
+    int B, H, T, D, W, dtype;
+    fibattn_opts o;
+    Call(const Tensor& q, const Tensor& k, int w, const Offsets& f, const Tensor& rk, const Tensor& res, PyObject* const* a) {
+        if (q.dim() != 4 || k.dim() < 2) value_error("q must be [B,H,T,D] and k [B,Hkv,T,D]");
+        B = (int)q.size(0); H = (int)q.size(1); T = (int)q.size(2); D = (int)q.size(3);
+        W = w;
+        const auto dt = q.scalar_type();
+        if (dt != at::kFloat && dt != at::kBFloat16) {
+            PyErr_Format(PyExc_TypeError, "unsupported dtype %s: fp32 or bf16", c10::toString(dt));
+            throw python_error();
+        }
+        dtype = dt == at::kFloat ? FIBATTN_F32 : FIBATTN_BF16;
+        if (rk.defined()) {
+            const auto want = k.scalar_type() == at::kBFloat16 ? at::kHalf : at::kFloat;
+            if (!(rk.is_cuda() && rk.is_contiguous() && rk.scalar_type() == want && rk.sizes() == k.sizes()))
+                value_error(want == at::kHalf ? "rotated_k must be a contiguous CUDA torch.float16 tensor of k's shape"
+                                              : "rotated_k must be a contiguous CUDA torch.float32 tensor of k's shape");
+        }
+        if (res.defined() && !(res.is_cuda() && res.is_contiguous() &&
+                               (size_t)(res.numel() * res.element_size()) >= fibattn_residual_bytes(B, H, T, D, W, f.K, dtype)))
+            value_error("residuals must be a contiguous CUDA buffer of residual_bytes(...) bytes");
+        o = fibattn_opts{};
+        o.rope_base = (float)as_float(a[0]);
+        o.scale = (float)as_float(a[1]);
+        o.no_dedup = PyObject_IsTrue(a[2]) ? 0 : 1;
+        o.round_offsets = PyObject_IsTrue(a[3]) ? 1 : 0;
+        o.Hkv = (int)k.size(1);
+        o.rotated_k = ptr(rk);
+        o.residuals = ptr(res);
+    }
+};
+
+void check_inputs(const Tensor& q, std::initializer_list<const Tensor*> ts, const char* msg) {
+    for (const Tensor* t : ts)
+        if (t->defined() && !(t->is_cuda() && t->is_contiguous() && t->scalar_type() == q.scalar_type())) value_error(msg);
+}
+
+Tensor like(const Tensor& given, const Tensor& t) { return given.defined() ? given : at::empty(t.sizes(), t.options()); }
+
+Tensor bytes(size_t need, const Tensor& q) {
+    return at::empty({(int64_t)std::max<size_t>(need, 256)}, q.options().dtype(at::kByte));
+}
+
+void* stream_of(PyObject* o) {
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    void* s = PyLong_AsVoidPtr(o);
+    if (!s && PyErr_Occurred()) throw python_error();
+    return s;
+}
+
+bool arity(Py_ssize_t n, Py_ssize_t want) {
+    if (n == want) return true;
+    PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
+    return false;
+}
+
+int call_fwd(const Call& c, const Tensor& q, const Tensor& k, const Tensor& v, const Tensor& out, const Tensor& lse,
+             const Tensor& ws, float alpha, const Offsets& f, void* st) {
+    void *pq = ptr(q), *pk = ptr(k), *pv = ptr(v), *po = ptr(out), *pl = ptr(lse), *pw = ptr(ws);
+    const size_t nw = ws.defined() ? (size_t)ws.numel() : 0;
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = fibattn_fwd(pq, pk, pv, po, static_cast<float*>(pl), c.B, c.H, c.T, c.D, c.W, alpha, f.f, f.K, c.dtype, &c.o, pw, nw, st);
+    Py_END_ALLOW_THREADS
+    return rc;
+}
+
+PyObject* tuple_of(std::initializer_list<const Tensor*> ts) {     // an undefined tensor is None
+    PyObject* r = PyTuple_New((Py_ssize_t)ts.size());
+    if (!r) return nullptr;
+    int i = 0;
+    for (const Tensor* t : ts) {
+        PyObject* x = Py_None;
+        if (t->defined()) x = THPVariable_Wrap(*t);
+        else Py_INCREF(Py_None);
+        PyTuple_SET_ITEM(r, i++, x);
+    }
+    return r;
+}
+
+const char kFwdInputs[] = "q, k, v must be contiguous CUDA tensors of one dtype";
+
+// fwd(q, k, v, offsets, W, alpha, rope_base, scale, dedup, round_offsets, kernel, out, lse, workspace, rotated_k,
+//     residuals, stream) -> (out, lse), or the call's status when it is not 0
+PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (!arity(n, 17)) return nullptr;
+    const Tensor &q = tensor(a[0], "q"), &k = tensor(a[1], "k"), &v = tensor(a[2], "v");
+    const Offsets f(a[3]);
+    const Tensor rk = optional(a[14], "rotated_k"), res = optional(a[15], "residuals");
+    Call c(q, k, (int)as_int(a[4]), f, rk, res, a + 6);
+    const float alpha = (float)as_float(a[5]);
+    c.o.fwd_kernel = (int)as_int(a[10]);
+    check_inputs(q, {&q, &k, &v}, kFwdInputs);
+    const Tensor out = like(optional(a[11], "out"), q);
+    Tensor lse = optional(a[12], "lse"), ws = optional(a[13], "workspace");
+    if (!lse.defined()) lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
+    // (a given workspace's size is checked by the library)
+    if (!ws.defined()) ws = bytes(fibattn_fwd_workspace_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype, &c.o), q);
+    const int rc = call_fwd(c, q, k, v, out, lse, ws, alpha, f, stream_of(a[16]));
+    return rc ? PyLong_FromLong(rc) : tuple_of({&out, &lse});
+    END_HANDLE_TH_ERRORS
+}
+
+// fwd_keep(q, k, v, offsets, W, alpha, rope_base, scale, dedup, round_offsets) -> (out, lse, rotated_k, residuals or
+// None): the forward of a training step on the current stream, with what its backward reads; residuals where the
+// tensor-core forward applies.  Or the call's status when it is not 0.
+PyObject* fwd_keep(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (!arity(n, 10)) return nullptr;
+    const Tensor &q = tensor(a[0], "q"), &k = tensor(a[1], "k"), &v = tensor(a[2], "v");
+    const Offsets f(a[3]);
+    Call c(q, k, (int)as_int(a[4]), f, Tensor(), Tensor(), a + 6);
+    const float alpha = (float)as_float(a[5]);
+    check_inputs(q, {&q, &k, &v}, kFwdInputs);
+    const Tensor out = at::empty(q.sizes(), q.options());
+    const Tensor lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
+    const Tensor rk = at::empty(k.sizes(), k.options().dtype(c.dtype == FIBATTN_BF16 ? at::kHalf : at::kFloat));
+    c.o.rotated_k = ptr(rk);
+    void* const st = stream_of(Py_None);
+    const size_t nr = fibattn_residual_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype);
+    Tensor res;
+    int rc = FIBATTN_ERR_UNSUPPORTED;
+    if (nr > 0) {
+        res = at::empty({(int64_t)nr}, q.options().dtype(at::kByte));
+        c.o.residuals = ptr(res);
+        rc = call_fwd(c, q, k, v, out, lse, Tensor(), alpha, f, st);
+    }
+    if (rc == FIBATTN_ERR_UNSUPPORTED) {
+        res = Tensor();
+        c.o.residuals = nullptr;
+        rc = call_fwd(c, q, k, v, out, lse, Tensor(), alpha, f, st);
+    }
+    return rc ? PyLong_FromLong(rc) : tuple_of({&out, &lse, &rk, &res});
+    END_HANDLE_TH_ERRORS
+}
+
+// bwd(q, k, v, offsets, W, alpha, rope_base, scale, dedup, round_offsets, kernel, out, lse, workspace, rotated_k,
+//     residuals, stream, dout, dq, dk, dv, dtheta, dd, rung_grads)
+//   -> (dq, dk, dv, dtheta [1] or None, dd [K] or None), or the call's status when it is not 0
+PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (!arity(n, 24)) return nullptr;
+    const Tensor &q = tensor(a[0], "q"), &k = tensor(a[1], "k"), &v = tensor(a[2], "v");
+    const Tensor &lse = tensor(a[12], "lse"), &dout = tensor(a[17], "dout");
+    const Offsets f(a[3]);
+    const Tensor rk = optional(a[14], "rotated_k"), res = optional(a[15], "residuals"), out = optional(a[11], "out");
+    Call c(q, k, (int)as_int(a[4]), f, rk, res, a + 6);
+    const float alpha = (float)as_float(a[5]);
+    c.o.bwd_kernel = (int)as_int(a[10]);
+    check_inputs(q, {&q, &k, &v, &dout, &out}, "q, k, v, dout, out must be contiguous CUDA tensors of one dtype");
+    const Tensor dq = like(optional(a[18], "dq"), q), dk = like(optional(a[19], "dk"), k), dv = like(optional(a[20], "dv"), v);
+    Tensor dth = optional(a[21], "dtheta"), dd = optional(a[22], "dd"), ws = optional(a[13], "workspace");
+    if (PyObject_IsTrue(a[23])) {
+        if (!dth.defined()) dth = at::empty({1}, q.options().dtype(at::kFloat));
+        if (!dd.defined()) dd = at::empty({std::max(f.K, 1)}, q.options().dtype(at::kFloat));
+    }
+    if (!ws.defined()) ws = bytes(fibattn_bwd_workspace_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype, &c.o), q);
+    void* const st = stream_of(a[16]);
+    void *pq = ptr(q), *pk = ptr(k), *pv = ptr(v), *po = ptr(out), *pl = ptr(lse), *pg = ptr(dout), *pw = ptr(ws);
+    void *pdq = ptr(dq), *pdk = ptr(dk), *pdv = ptr(dv), *pth = ptr(dth), *pdd = ptr(dd);
+    const size_t nw = (size_t)ws.numel();
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = fibattn_bwd(pq, pk, pv, po, static_cast<const float*>(pl), pg, pdq, pdk, pdv, static_cast<float*>(pth),
+                     static_cast<float*>(pdd), c.B, c.H, c.T, c.D, c.W, alpha, f.f, f.K, c.dtype, &c.o, pw, nw, st);
+    Py_END_ALLOW_THREADS
+    if (rc) return PyLong_FromLong(rc);
+    if (dth.defined() && !(dth.dim() == 1 && dth.size(0) == 1)) dth = dth.slice(0, 0, 1);
+    if (dd.defined() && !(dd.dim() == 1 && dd.size(0) == f.K)) dd = dd.slice(0, 0, f.K);
+    return tuple_of({&dq, &dk, &dv, &dth, &dd});
+    END_HANDLE_TH_ERRORS
+}
+
+// alpha_of_theta(theta) -> 0.5 + sigmoid(theta), as the library computes it
+PyObject* alpha_of_theta(PyObject*, PyObject* o) {
+    HANDLE_TH_ERRORS
+    const float th = (float)as_float(o);
+    float al = 0.f;
+    const int rc = fibattn_alpha_schedule(1, 1, &th, 0, &al);
+    if (rc) value_error(fibattn_last_error());
+    return PyFloat_FromDouble(al);
+    END_HANDLE_TH_ERRORS
+}
+
+PyMethodDef methods[] = {
+    {"fwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(fwd)), METH_FASTCALL, nullptr},
+    {"fwd_keep", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(fwd_keep)), METH_FASTCALL, nullptr},
+    {"bwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(bwd)), METH_FASTCALL, nullptr},
+    {"alpha_of_theta", alpha_of_theta, METH_O, nullptr},
+    {nullptr, nullptr, 0, nullptr},
+};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "fibattn_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit_fibattn_marshal() { return PyModule_Create(&module); }
