@@ -186,7 +186,7 @@ __device__ __forceinline__ void key_pass(float (&acc)[8][4], const float* X, con
 // passes of its tile.
 template <int NT, bool SPLIT>
 __global__ void __launch_bounds__(kWarps * 32, 2)
-bwd_key_mma_kernel(const __grid_constant__ RowMaps tmQ, const __grid_constant__ RowMaps tmG, BwdArgs a,
+bwd_key_mma_kernel(const __grid_constant__ BoxMaps tmQ, const __grid_constant__ BoxMaps tmG, BwdArgs a,
                    MmaLayout L) {
     // The kernel before this one is the query pass of the same call.  With the
     // forward residuals pass 0 reads only p and dO, which it does not write,
@@ -246,8 +246,11 @@ bwd_key_mma_kernel(const __grid_constant__ RowMaps tmQ, const __grid_constant__ 
             const int qhead = b * s.H + hk * s.G + g;
             const float* X = (pass ? a.DSs : a.Ps) + (size_t)qhead * a.S * s.T;
             if (warp == 0) {
-                const RowMaps& m = pass ? tmQ : tmG;
-                issue_rows(buf, &m.m64, &m.m8, L, j0, qhead, &bar, lane);
+                const BoxMaps& m = pass ? tmQ : tmG;
+                if (lane == 0) mbar_expect_tx(&bar, L.box_bytes);
+                __syncwarp();
+                if constexpr (NT == 4) issue_rows(sbase, m, L, j0, qhead, &bar, lane);
+                else if (lane == 0) issue_boxes(sbase, m, L, j0, qhead, &bar);
             }
             if (pass == 0)
                 key_pass<NT>(acc, X, a, L, sbase, bw, wrel, g4, c4, lane, vlo, vhi, &bar, parity, ok,
@@ -329,7 +332,7 @@ bwd_key_mma_kernel(const __grid_constant__ RowMaps tmQ, const __grid_constant__ 
 }
 
 template <int NT>
-cudaError_t launch_nt(const RowMaps& mq, const RowMaps& mg, const BwdArgs& a, const MmaLayout& L,
+cudaError_t launch_nt(const BoxMaps& mq, const BoxMaps& mg, const BwdArgs& a, const MmaLayout& L,
                       unsigned grid, size_t smem, cudaStream_t st) {
     // one block per tile unless that leaves the GPU under two waves of blocks
     static int slots = 0;
@@ -364,10 +367,10 @@ int bwd_key_mma_blocks(const Shape& s) {
 cudaError_t launch_bwd_key_mma(const BwdArgs& a, const MmaLayout& L, cudaStream_t st) {
     const long long grid = bwd_key_mma_blocks(a.s);
     if (grid <= 0) return cudaSuccess;
-    RowMaps mq, mg;
+    BoxMaps mq, mg;
     const int heads = a.s.B * a.s.H;
-    if (!encode_row_maps(&mq, a.qt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.s.T, heads) ||
-        !encode_row_maps(&mg, a.dout, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.s.T, heads))
+    if (!encode_box_maps(&mq, a.qt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.s.T, heads) ||
+        !encode_box_maps(&mg, a.dout, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.s.T, heads))
         return cudaErrorInvalidValue;
     const size_t smem = bwd_key_mma_smem_bytes(L, a.saved != 0);
     switch (L.nt) {

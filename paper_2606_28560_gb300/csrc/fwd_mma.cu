@@ -27,7 +27,7 @@
 //
 // Staging: the CTA's union of key rows (rotated keys, fp16) and then of value
 // rows (bf16, same buffer) is copied by TMA (3-D tensor maps [heads][T][64],
-// 64-row boxes with 8-row tails, 128-byte swizzle, rows outside [0, T)
+// 64- and 32-row boxes, 128-byte swizzle, rows outside [0, T)
 // zero-filled) under mbarriers with bounded waits; the value copies are
 // issued by the last warp done with the keys.  The one-head form writes its
 // output rows (and the rotated query rows it keeps) through a 1 KB stage per
@@ -63,7 +63,7 @@ constexpr int kRowsPerWarp = 15;                 // useful query rows of a 16-ro
 // the far-minus-floor raw score of every rung and 1 / (row sum) per query.
 template <int NT, int TEAMS, bool SAVE>
 __global__ void __launch_bounds__(kWarps * 32 * TEAMS, TEAMS == 1 ? 2 : 1)
-fwd_mma_kernel(const __grid_constant__ RowMaps tmK, const __grid_constant__ RowMaps tmV,
+fwd_mma_kernel(const __grid_constant__ BoxMaps tmK, const __grid_constant__ BoxMaps tmV,
                FwdArgs a, MmaLayout L) {
     // The kernel before this one is the key rotation of the same call, which
     // writes only the rotated keys: the query rows are loaded before waiting
@@ -122,11 +122,17 @@ fwd_mma_kernel(const __grid_constant__ RowMaps tmK, const __grid_constant__ RowM
         mbar_init(&bars[1], 1);
         keys_done = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        mbar_expect_tx(&bars[0], L.box_bytes);
+        mbar_expect_tx(&bars[1], L.box_bytes);
     }
     __syncthreads();                              // barrier init visible
+    auto issue = [&](unsigned dst, const BoxMaps& m, unsigned long long* bar) {
+        if constexpr (SAVE && NT == 4) issue_rows(dst, m, L, i0, head, bar, lane);
+        else if (lane == 0) issue_boxes(dst, m, L, i0, head, bar);
+    };
     if (tid < 32) {
-        issue_rows(buf, &tmK.m64, &tmK.m8, L, i0, head, &bars[0], lane);
-        if (TEAMS == 2) issue_rows(vbuf, &tmV.m64, &tmV.m8, L, i0, head, &bars[1], lane);
+        issue(sbase, tmK, &bars[0]);
+        if (TEAMS == 2) issue(vbase, tmV, &bars[1]);
     }
     // A warp whose tile starts past the end of the sequence (the last tile of
     // a head) has no query to compute; in the one-head form it still counts
@@ -139,7 +145,7 @@ fwd_mma_kernel(const __grid_constant__ RowMaps tmK, const __grid_constant__ RowM
             before = __shfl_sync(0xffffffffu, before, 0);
             if (before == kWarps - 1) {
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                issue_rows(buf, &tmV.m64, &tmV.m8, L, i0, head, &bars[1], lane);
+                issue(sbase, tmV, &bars[1]);
             }
         }
         return;
@@ -405,7 +411,7 @@ fwd_mma_kernel(const __grid_constant__ RowMaps tmK, const __grid_constant__ RowM
         before = __shfl_sync(0xffffffffu, before, 0);
         if (before == kWarps - 1) {
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            issue_rows(buf, &tmV.m64, &tmV.m8, L, i0, head, &bars[1], lane);
+            issue(sbase, tmV, &bars[1]);
         }
     }
 
@@ -592,7 +598,7 @@ fwd_mma_kernel(const __grid_constant__ RowMaps tmK, const __grid_constant__ RowM
 // ------------------------------------------------------------ host side ----
 
 template <int NT, int TEAMS>
-cudaError_t launch_nt(const RowMaps& mk, const RowMaps& mv, const FwdArgs& a, const MmaLayout& L,
+cudaError_t launch_nt(const BoxMaps& mk, const BoxMaps& mv, const FwdArgs& a, const MmaLayout& L,
                       unsigned grid, size_t smem, cudaStream_t st) {
     // (the grouped form runs only without residuals)
     auto kern = a.res_P ? fwd_mma_kernel<NT, TEAMS, TEAMS == 1> : fwd_mma_kernel<NT, TEAMS, false>;
@@ -664,6 +670,37 @@ void layout_intervals(Iv* iv, int n, MmaLayout* L) {
         rows += len;
     }
     L->rows = rows;
+}
+
+// The copies of the merged intervals (every one at least 121 rows long): whole
+// 64-row boxes, then for the rest one box of 32 or 64 rows that ends with the
+// interval.  False when the list would not hold them.
+bool plan_boxes(MmaLayout* L) {
+    int n = 0;
+    L->box_bytes = 0;
+    for (int h = 64; h >= 32; h -= 32) {
+        for (int iv = 0; iv < L->n_iv; ++iv) {
+            const int len = L->iv_len[iv], full = len / 64, rest = len % 64;
+            auto box = [&](int r) {
+                if (n == kMmaMaxBoxes) return false;
+                L->box_smem[n] = (short)(L->iv_smem[iv] + r);
+                L->box_row[n] = L->iv_start[iv] + r;
+                ++n;
+                L->box_bytes += (unsigned)h * 128u;
+                return true;
+            };
+            if (h == 64) {
+                for (int i = 0; i < full; ++i)
+                    if (!box(64 * i)) return false;
+                if (rest > 32 && !box(len - 64)) return false;
+            } else if (rest > 0 && rest <= 32) {
+                if (!box(len - 32)) return false;
+            }
+        }
+        if (h == 64) L->n_box64 = n;
+    }
+    L->n_box = n;
+    return true;
 }
 
 int smem_row_of(const MmaLayout& L, int rel) {
@@ -763,7 +800,7 @@ bool build_mma_layout(const Shape& s, const RungParams& r, double rope_base, siz
     L->bytes_lo = (unsigned)L->rows * 128u;
     L->bytes_hi = 0;
     if (reserve_rows > 0) plan_tile_regions(L, reserve_rows);
-    return fwd_mma_smem_bytes(*L) <= smem_limit;
+    return plan_boxes(L) && fwd_mma_smem_bytes(*L) <= smem_limit;
 }
 
 bool build_key_layout(const Shape& s, const RungParams& r, double rope_base, size_t smem_limit, MmaLayout* L) {
@@ -790,16 +827,16 @@ bool build_key_layout(const Shape& s, const RungParams& r, double rope_base, siz
     L->lo_start = 0;
     L->bytes_lo = (unsigned)L->rows * 128u;
     L->bytes_hi = 0;
-    return fwd_mma_smem_bytes(*L) <= smem_limit;
+    return plan_boxes(L) && fwd_mma_smem_bytes(*L) <= smem_limit;
 }
 
 cudaError_t launch_fwd_mma(const FwdArgs& a, const MmaLayout& L, cudaStream_t st) {
     const long long tiles = (a.s.T + kMmaTile - 1) / kMmaTile;
-    RowMaps mk, mv;
+    BoxMaps mk, mv;
     const int heads = a.s.B * a.s.Hkv;
     if (tiles * a.s.B * a.s.H <= 0) return cudaSuccess;
-    if (!encode_row_maps(&mk, a.kt, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, a.s.T, heads) ||
-        !encode_row_maps(&mv, a.v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.s.T, heads))
+    if (!encode_box_maps(&mk, a.kt, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, a.s.T, heads) ||
+        !encode_box_maps(&mv, a.v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a.s.T, heads))
         return cudaErrorInvalidValue;
     // Grouped-query attention: one CTA per kv head's tile with both staged
     // tensors resident, when they fit and no residuals are written (with the

@@ -9,6 +9,7 @@ namespace fibattn {
 constexpr int kMmaWarps = 8;                      // one 16-row MMA tile per warp
 constexpr int kMmaTile = kMmaWarps * 15;          // queries per CTA (tiles every 15 rows)
 constexpr int kMmaMaxRungs = 16;
+constexpr int kMmaMaxBoxes = 48;                  // 1816 rows (227 KB) in 17 intervals: at most 28 + 17 boxes
 
 // Rows a CTA stages, relative to its first query: merged intervals of the
 // window band [-Wp, M+1) and the rung slabs [-s0-1, M+1-s0), each rounded up
@@ -42,6 +43,14 @@ struct MmaLayout {
     int buf_rows;
     int lo_start;
     unsigned bytes_lo, bytes_hi;
+    // The same rows as a flat list of copies: boxes [0, n_box64) of 64 rows,
+    // boxes [n_box64, n_box) of 32.  A box's first shared row and first relative
+    // row; an interval's last box ends where it ends and may repeat rows of
+    // the one before.  box_bytes: what all of them deliver.
+    int n_box64, n_box;
+    unsigned box_bytes;
+    short box_smem[kMmaMaxBoxes];
+    int box_row[kMmaMaxBoxes];
 };
 
 constexpr int kTileRows = 128;                    // a tile's own rows of one tensor (two 64-row boxes)
@@ -67,6 +76,11 @@ bool encode_rows_map(CUtensorMap* map, const void* base, CUtensorMapDataType dt,
 struct RowMaps { CUtensorMap m64, m8; };
 inline bool encode_row_maps(RowMaps* m, const void* base, CUtensorMapDataType dt, int T, int heads) {
     return encode_rows_map(&m->m64, base, dt, T, heads, 64) && encode_rows_map(&m->m8, base, dt, T, heads, 8);
+}
+// The same rows as 64-row and as 32-row boxes (MmaLayout::box_row).
+struct BoxMaps { CUtensorMap m64, m32; };
+inline bool encode_box_maps(BoxMaps* m, const void* base, CUtensorMapDataType dt, int T, int heads) {
+    return encode_rows_map(&m->m64, base, dt, T, heads, 64) && encode_rows_map(&m->m32, base, dt, T, heads, 32);
 }
 // The query backward's tile rows: q, dO, o (64-row loads) and the rotated q
 // it writes back (40-row stores).

@@ -56,6 +56,12 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
         }
     }
 }
+__device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map, int x, int y, int z,
+                                            unsigned long long* bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+                 " [%0], [%1, {%2, %3, %4}], [%5];\n"
+                 :: "r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z,
                                             unsigned long long* bar) {
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
@@ -142,26 +148,43 @@ __device__ __forceinline__ unsigned row_chunk(unsigned base, int row, int ch) {
     return base + ((unsigned)row << 7) + ((unsigned)((row ^ ch) & 7) << 4);
 }
 
-// Warp 0 issues the copies of one staged tensor.  Lane n copies merged
-// interval n: whole 64-row boxes (map64) first, then 8-row boxes (map8) for
-// the rest of it (interval lengths are multiples of 8 rows).  Large boxes move
-// the same rows at well over the rate of 8-row ones.  Lane 0 announces the
-// byte count before any copy is issued.
-__device__ __forceinline__ void issue_rows(unsigned char* dst, const CUtensorMap* map64, const CUtensorMap* map8,
-                                           const MmaLayout& L, int i0, int head, unsigned long long* bar, int lane) {
-    if (lane == 0) mbar_expect_tx(bar, (unsigned)L.rows * 128u);
-    __syncwarp();
+// The copies of a staged tensor.  How they are issued is on a CTA's critical
+// path (100 more instructions ahead of them cost the forward 8 %), and they
+// go out one after another, so they are few: per merged interval whole 64-row
+// boxes, and for the rest of it one box of 32 or 64 rows that ends with the
+// interval and repeats rows of the box before (8-row boxes made up to seven of
+// that rest).  Forward B4 T4096 W10 40.5 -> 38.4 us a call; training layer B16
+// T1024 133.6 -> 131.7, with two kv heads 127.1 -> 124.2, B2 T16384 pow2 227.7
+// -> 223.4.  Two forms, for kernels that the compiler schedules differently
+// around them (NT = 4 with residuals: 84.3 us lane by lane, 88.3 from the list;
+// NT = 3 without: 39.7 and 37.2; issued by all eight warps: slower than by
+// one).  Both deliver L.box_bytes, with which somebody arms the barrier in the
+// same phase.
+//
+// issue_boxes: one thread, from the host's flat list.
+__device__ __forceinline__ void issue_boxes(unsigned dst, const BoxMaps& m, const MmaLayout& L, int i0, int head,
+                                            unsigned long long* bar) {
+    for (int b = 0; b < L.n_box; ++b)
+        tma_load_3d(dst + (unsigned)L.box_smem[b] * 128u, b < L.n_box64 ? &m.m64 : &m.m32, 0, i0 + L.box_row[b], head, bar);
+}
+// issue_rows: one warp, lane n copies merged interval n.
+__device__ __forceinline__ void issue_rows(unsigned dst, const BoxMaps& m, const MmaLayout& L, int i0, int head,
+                                           unsigned long long* bar, int lane) {
     for (int iv = lane; iv < L.n_iv; iv += 32) {
         const int len = L.iv_len[iv], srow = L.iv_smem[iv], grow = i0 + L.iv_start[iv];
         int r = 0;
-        for (; r + 64 <= len; r += 64) tma_load_3d(dst + (size_t)(srow + r) * 128, map64, 0, grow + r, head, bar);
-        for (; r < len; r += 8) tma_load_3d(dst + (size_t)(srow + r) * 128, map8, 0, grow + r, head, bar);
+        for (; r + 64 <= len; r += 64) tma_load_3d(dst + (unsigned)(srow + r) * 128u, &m.m64, 0, grow + r, head, bar);
+        if (r + 32 < len) tma_load_3d(dst + (unsigned)(srow + len - 64) * 128u, &m.m64, 0, grow + len - 64, head, bar);
+        else if (r < len) tma_load_3d(dst + (unsigned)(srow + len - 32) * 128u, &m.m32, 0, grow + len - 32, head, bar);
     }
 }
 
-// One batch of the copies issue_rows makes: boxes that start at or after
+// One batch of a staged tensor's copies: boxes that start at or after
 // L.lo_start (hi_batch false) or before it (hi_batch true); the barrier
-// expects that batch's bytes.  Boxes are the same as issue_rows's.
+// expects that batch's bytes.  Lane n copies merged interval n: whole 64-row
+// boxes (map64) first, then 8-row boxes (map8) for the rest of it (interval
+// lengths are multiples of 8 rows).  Lane 0 announces the byte count before
+// any copy is issued.
 __device__ __forceinline__ void issue_rows_batch(unsigned char* dst, const CUtensorMap* map64, const CUtensorMap* map8,
                                                  const MmaLayout& L, int i0, int head, unsigned long long* bar,
                                                  int lane, bool hi_batch) {
