@@ -82,7 +82,10 @@ __device__ __forceinline__ void key_pass(float (&acc)[8][4], const float* X, con
         const int i = u >> 4, x = u & 15;
         const int q = bw + L.act_s0[i] + x;
         const bool use = i < L.n_act && q < s.T;
-        rvv[j] = use ? X[(unsigned)((s.W + 1 + L.act_k[i]) * s.T + q)] : 0.f;
+        // (NT = 4 from the host's row offsets, 94.9 -> 92.8 us at B2 T16384; the
+        // NT = 3 kernel is 1 % slower with them)
+        const unsigned row = NT == 4 ? (unsigned)L.act_row[i] : (unsigned)((s.W + 1 + L.act_k[i]) * s.T);
+        rvv[j] = use ? X[row + (unsigned)q] : 0.f;
     }
     if (IL) {
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -155,8 +158,12 @@ __device__ __forceinline__ void key_pass(float (&acc)[8][4], const float* X, con
     // Rungs whose slab starts before the end of the sequence: a prefix of the
     // list.  Two per iteration (independent work to overlap); an odd count
     // runs one padding entry, whose values are zero.
+    // (Counted over all entries at once: a loop to the first that fails waits for
+    // a parameter load each time; 47.1 -> 45.1 us at B16 T1024, 98.3 -> 94.9 at
+    // B2 T16384.)
     int n_use = 0;
-    while (n_use < L.n_act && bw + L.act_s0[n_use] < s.T) ++n_use;
+#pragma unroll
+    for (int i = 0; i < kMmaMaxRungs; ++i) n_use += i < L.n_act && bw + L.act_s0[i] < s.T;
 #pragma unroll 1
     for (int i = 0; i < n_use; i += 2) {
 #pragma unroll
