@@ -268,15 +268,15 @@ def step_method_bytes():
 # lines only: comments and blank lines are left out): once the code of a file
 # of the kernel changes, the figure is reported as null until the next capture.
 NCU_TRAFFIC = {
-    "bwd_query_mma": {"bytes_at_b32": 165865728 + 34423040,
+    "bwd_query_mma": {"bytes_at_b32": 165826560 + 34649856,
                       "sources": ("bwd_mma.cu", "mma_common.cuh", "fwd_mma.cuh", "fibattn_internal.cuh"),
-                      "sha256": "b200e61a7c2718d93368c317cf0bc8c056fae5f1aeb7699de3da502589b892ee"},
-    "bwd_key_mma": {"bytes_at_b32": 104528640 + 36358400,
+                      "sha256": "21821344fbc102b8f92e80482f8298a1532983e746753a7c0afda5a66c384805"},
+    "bwd_key_mma": {"bytes_at_b32": 104474112 + 36254464,
                     "sources": ("bwd_key_mma.cu", "mma_common.cuh", "fwd_mma.cuh", "fibattn_internal.cuh"),
-                    "sha256": "73f3bd8d30f5d7b450147f07b9118be3981338e5afd560b7cbc599c314caa730"},
-    "fwd": {"bytes_at_b32": 100805632 + 57507584,
+                    "sha256": "765280ce807e12c46e3220248e7348fa6ab252fc81245b85f9100b562971ea78"},
+    "fwd": {"bytes_at_b32": 100809216 + 57611264,
             "sources": ("fwd_mma.cu", "mma_common.cuh", "fwd_mma.cuh", "fibattn_internal.cuh"),
-            "sha256": "69c9b864ca4eec6a2feb267f6b72a25de32b0681fa874692afc5e807f9d29d48"},
+            "sha256": "0924d8b3132882c710ecea13e495835180fd9a518aa9aa5d5fe907f97b44bf4a"},
 }
 
 
