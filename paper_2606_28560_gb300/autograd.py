@@ -62,10 +62,12 @@ def _attend(q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha):
     for: it then keeps nothing for a backward (the residuals add half again to
     the forward's traffic) and autograd takes no part.  A call inside a
     function transform or forward-mode differentiation goes to autograd, which
-    refuses it."""
+    refuses it; so does a call that is being traced, whose record is then the
+    Function (of the native call it would hold only the output's allocation)."""
     alpha = None if alpha is None else float(alpha)
     if (torch.is_grad_enabled() and (q.requires_grad or k.requires_grad or v.requires_grad or theta.requires_grad)) \
-            or torch._C._are_functorch_transforms_active() or torch.autograd.forward_ad._current_level >= 0:
+            or torch._C._are_functorch_transforms_active() or torch.autograd.forward_ad._current_level >= 0 \
+            or torch.jit.is_tracing():
         return FibAttentionFunction.apply(q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha)
     if alpha is None:
         alpha = alpha_of_theta(float(theta))
