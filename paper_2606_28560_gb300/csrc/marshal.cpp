@@ -7,6 +7,7 @@
 
 #include <ATen/core/Tensor.h>
 #include <ATen/ops/empty.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -74,11 +75,11 @@ struct Call {
         dtype = dt == at::kFloat ? FIBATTN_F32 : FIBATTN_BF16;
         if (rk.defined()) {
             const auto want = k.scalar_type() == at::kBFloat16 ? at::kHalf : at::kFloat;
-            if (!(rk.is_cuda() && rk.is_contiguous() && rk.scalar_type() == want && rk.sizes() == k.sizes()))
+            if (!(rk.is_cuda() && rk.device() == q.device() && rk.is_contiguous() && rk.scalar_type() == want && rk.sizes() == k.sizes()))
                 value_error(want == at::kHalf ? "rotated_k must be a contiguous CUDA torch.float16 tensor of k's shape"
                                               : "rotated_k must be a contiguous CUDA torch.float32 tensor of k's shape");
         }
-        if (res.defined() && !(res.is_cuda() && res.is_contiguous() &&
+        if (res.defined() && !(res.is_cuda() && res.device() == q.device() && res.is_contiguous() &&
                                (size_t)(res.numel() * res.element_size()) >= fibattn_residual_bytes(B, H, T, D, W, f.K, dtype)))
             value_error("residuals must be a contiguous CUDA buffer of residual_bytes(...) bytes");
         o = fibattn_opts{};
@@ -92,9 +93,29 @@ struct Call {
     }
 };
 
+// The library sees pointers and the extents of q (and k's heads): whatever it
+// reads or writes through the others is checked to be there, before any launch.
 void check_inputs(const Tensor& q, std::initializer_list<const Tensor*> ts, const char* msg) {
     for (const Tensor* t : ts)
         if (t->defined() && !(t->is_cuda() && t->is_contiguous() && t->scalar_type() == q.scalar_type())) value_error(msg);
+    for (const Tensor* t : ts)
+        if (t->defined() && t->device() != q.device()) value_error("the tensors of a call must be on one device");
+}
+void check_kv(const Tensor& q, const Tensor& k, const Tensor& v) {
+    const int64_t n = q.size(0) * k.size(1) * q.size(2) * q.size(3);
+    if (k.numel() != n || v.numel() != n) value_error("k and v must be [B,Hkv,T,D], with q's B, T and D");
+}
+// A buffer of the caller's: n entries of type dt (more are allowed).
+void check_buffer(const Tensor& t, const Tensor& q, at::ScalarType dt, int64_t n, const char* name) {
+    if (!t.defined() || (t.numel() >= n && t.scalar_type() == dt && t.is_contiguous() && t.device() == q.device())) return;
+    PyErr_Format(PyExc_ValueError, "%s must be contiguous, %s, on q's device and hold %lld entries", name,
+                 c10::toString(dt), (long long)n);
+    throw python_error();
+}
+// (its size is checked by the library)
+void check_workspace(const Tensor& ws, const Tensor& q) {
+    if (ws.defined() && !(ws.is_contiguous() && ws.device() == q.device()))
+        value_error("workspace must be contiguous and on q's device");
 }
 
 Tensor like(const Tensor& given, const Tensor& t) { return given.defined() ? given : at::empty(t.sizes(), t.options()); }
@@ -153,11 +174,16 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     Call c(q, k, (int)as_int(a[4]), f, rk, res, a + 6);
     const float alpha = (float)as_float(a[5]);
     c.o.fwd_kernel = (int)as_int(a[10]);
-    check_inputs(q, {&q, &k, &v}, kFwdInputs);
-    const Tensor out = like(optional(a[11], "out"), q);
+    const Tensor given = optional(a[11], "out");
     Tensor lse = optional(a[12], "lse"), ws = optional(a[13], "workspace");
+    check_kv(q, k, v);
+    check_buffer(given, q, q.scalar_type(), q.numel(), "out");
+    check_buffer(lse, q, at::kFloat, q.size(0) * q.size(1) * q.size(2), "lse");
+    check_workspace(ws, q);
+    check_inputs(q, {&q, &k, &v}, kFwdInputs);
+    const c10::cuda::CUDAGuard device(q.device());
+    const Tensor out = like(given, q);
     if (!lse.defined()) lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
-    // (a given workspace's size is checked by the library)
     if (!ws.defined()) ws = bytes(fibattn_fwd_workspace_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype, &c.o), q);
     const int rc = call_fwd(c, q, k, v, out, lse, ws, alpha, f, stream_of(a[16]));
     return rc ? PyLong_FromLong(rc) : tuple_of({&out, &lse});
@@ -174,7 +200,9 @@ PyObject* fwd_keep(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const Offsets f(a[3]);
     Call c(q, k, (int)as_int(a[4]), f, Tensor(), Tensor(), a + 6);
     const float alpha = (float)as_float(a[5]);
+    check_kv(q, k, v);
     check_inputs(q, {&q, &k, &v}, kFwdInputs);
+    const c10::cuda::CUDAGuard device(q.device());
     const Tensor out = at::empty(q.sizes(), q.options());
     const Tensor lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
     const Tensor rk = at::empty(k.sizes(), k.options().dtype(c.dtype == FIBATTN_BF16 ? at::kHalf : at::kFloat));
@@ -210,9 +238,21 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     Call c(q, k, (int)as_int(a[4]), f, rk, res, a + 6);
     const float alpha = (float)as_float(a[5]);
     c.o.bwd_kernel = (int)as_int(a[10]);
-    check_inputs(q, {&q, &k, &v, &dout, &out}, "q, k, v, dout, out must be contiguous CUDA tensors of one dtype");
-    const Tensor dq = like(optional(a[18], "dq"), q), dk = like(optional(a[19], "dk"), k), dv = like(optional(a[20], "dv"), v);
+    Tensor dq = optional(a[18], "dq"), dk = optional(a[19], "dk"), dv = optional(a[20], "dv");
     Tensor dth = optional(a[21], "dtheta"), dd = optional(a[22], "dd"), ws = optional(a[13], "workspace");
+    check_kv(q, k, v);
+    if (dout.numel() != q.numel()) value_error("dout must be of q's shape");
+    check_buffer(out, q, q.scalar_type(), q.numel(), "out");
+    check_buffer(lse, q, at::kFloat, q.size(0) * q.size(1) * q.size(2), "lse");
+    check_buffer(dq, q, q.scalar_type(), q.numel(), "dq");
+    check_buffer(dk, q, q.scalar_type(), k.numel(), "dk");
+    check_buffer(dv, q, q.scalar_type(), k.numel(), "dv");
+    check_buffer(dth, q, at::kFloat, 1, "dtheta");
+    check_buffer(dd, q, at::kFloat, f.K, "dd");
+    check_workspace(ws, q);
+    check_inputs(q, {&q, &k, &v, &dout, &out}, "q, k, v, dout, out must be contiguous CUDA tensors of one dtype");
+    const c10::cuda::CUDAGuard device(q.device());
+    dq = like(dq, q); dk = like(dk, k); dv = like(dv, v);
     if (PyObject_IsTrue(a[23])) {
         if (!dth.defined()) dth = at::empty({1}, q.options().dtype(at::kFloat));
         if (!dd.defined()) dd = at::empty({std::max(f.K, 1)}, q.options().dtype(at::kFloat));
