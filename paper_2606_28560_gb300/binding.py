@@ -291,7 +291,10 @@ def fwd(q, k, v, alpha: float, offsets, W: int, *, rope_base=1e4, scale=None, de
     rotated keys for a later ``bwd(..., rotated_k=...)``.  ``residuals``:
     optional buffer (``residuals_like(q, W, K)``) that receives the rotated
     queries, p of every slot and the rung score differences for a later
-    ``bwd(..., residuals=...)`` (tensor-core forward only).  Returns (out, lse)."""
+    ``bwd(..., residuals=...)`` (tensor-core forward only).  ``stream``: the
+    stream of the kernels in place of the current one; what the call allocates
+    is safe on both, the tensors it is given have to live until that stream is
+    done with them.  Returns (out, lse)."""
     r = (_marshal_module or _marshal()).fwd(
         q, k, v, _offsets(offsets), int(W), alpha, rope_base, scale or 0.0, dedup, round_offsets, FWD_KERNELS[kernel], out,
         lse, workspace, rotated_k, residuals, None if stream is None else stream.cuda_stream)

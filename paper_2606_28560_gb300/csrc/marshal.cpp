@@ -9,6 +9,7 @@
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
+#include <cuda_runtime_api.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -124,12 +125,30 @@ Tensor bytes(size_t need, const Tensor& q) {
     return at::empty({(int64_t)std::max<size_t>(need, 256)}, q.options().dtype(at::kByte));
 }
 
-void* stream_of(PyObject* o) {
-    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-    void* s = PyLong_AsVoidPtr(o);
-    if (!s && PyErr_Occurred()) throw python_error();
-    return s;
-}
+// The stream of a call: the current one, or the caller's.  Memory allocated
+// while it stands comes from that stream's pool: a workspace released on return
+// is reused by later work of the same stream only, where the current stream's
+// next allocation could have had it while the kernels still ran.
+struct OnStream {
+    const c10::cuda::CUDAStream current;
+    cudaStream_t st;
+    c10::cuda::OptionalCUDAStreamGuard guard;
+    explicit OnStream(PyObject* o) : current(c10::cuda::getCurrentCUDAStream()), st(current.stream()) {
+        if (o == Py_None) return;
+        st = static_cast<cudaStream_t>(PyLong_AsVoidPtr(o));
+        if (!st && PyErr_Occurred()) throw python_error();
+        const cudaStream_t pool = st == cudaStreamLegacy ? nullptr : st;      // (two names of the default stream)
+        if (pool != current.stream())
+            guard.reset_stream(pool ? c10::cuda::getStreamFromExternal(pool, current.device_index())
+                                    : c10::cuda::getDefaultCUDAStream(current.device_index()));
+    }
+    // Results made here are the caller's, who may use and drop them on the current stream.
+    void results(std::initializer_list<std::pair<const Tensor*, bool>> ts) const {
+        if (!guard.current_stream()) return;
+        for (const auto& [t, made] : ts)
+            if (made && t->defined()) t->record_stream(current);
+    }
+};
 
 bool arity(Py_ssize_t n, Py_ssize_t want) {
     if (n == want) return true;
@@ -182,10 +201,13 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_workspace(ws, q);
     check_inputs(q, {&q, &k, &v}, kFwdInputs);
     const c10::cuda::CUDAGuard device(q.device());
+    const OnStream on(a[16]);
     const Tensor out = like(given, q);
+    const bool own_lse = !lse.defined();
     if (!lse.defined()) lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
     if (!ws.defined()) ws = bytes(fibattn_fwd_workspace_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype, &c.o), q);
-    const int rc = call_fwd(c, q, k, v, out, lse, ws, alpha, f, stream_of(a[16]));
+    const int rc = call_fwd(c, q, k, v, out, lse, ws, alpha, f, on.st);
+    on.results({{&out, !given.defined()}, {&lse, own_lse}});
     return rc ? PyLong_FromLong(rc) : tuple_of({&out, &lse});
     END_HANDLE_TH_ERRORS
 }
@@ -207,7 +229,7 @@ PyObject* fwd_keep(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const Tensor lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
     const Tensor rk = at::empty(k.sizes(), k.options().dtype(c.dtype == FIBATTN_BF16 ? at::kHalf : at::kFloat));
     c.o.rotated_k = ptr(rk);
-    void* const st = stream_of(Py_None);
+    void* const st = c10::cuda::getCurrentCUDAStream().stream();
     const size_t nr = fibattn_residual_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype);
     Tensor res;
     int rc = FIBATTN_ERR_UNSUPPORTED;
@@ -252,21 +274,23 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_workspace(ws, q);
     check_inputs(q, {&q, &k, &v, &dout, &out}, "q, k, v, dout, out must be contiguous CUDA tensors of one dtype");
     const c10::cuda::CUDAGuard device(q.device());
+    const OnStream on(a[16]);
+    const bool own[5] = {!dq.defined(), !dk.defined(), !dv.defined(), !dth.defined(), !dd.defined()};
     dq = like(dq, q); dk = like(dk, k); dv = like(dv, v);
     if (PyObject_IsTrue(a[23])) {
         if (!dth.defined()) dth = at::empty({1}, q.options().dtype(at::kFloat));
         if (!dd.defined()) dd = at::empty({std::max(f.K, 1)}, q.options().dtype(at::kFloat));
     }
     if (!ws.defined()) ws = bytes(fibattn_bwd_workspace_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype, &c.o), q);
-    void* const st = stream_of(a[16]);
     void *pq = ptr(q), *pk = ptr(k), *pv = ptr(v), *po = ptr(out), *pl = ptr(lse), *pg = ptr(dout), *pw = ptr(ws);
     void *pdq = ptr(dq), *pdk = ptr(dk), *pdv = ptr(dv), *pth = ptr(dth), *pdd = ptr(dd);
     const size_t nw = (size_t)ws.numel();
     int rc;
     Py_BEGIN_ALLOW_THREADS
     rc = fibattn_bwd(pq, pk, pv, po, static_cast<const float*>(pl), pg, pdq, pdk, pdv, static_cast<float*>(pth),
-                     static_cast<float*>(pdd), c.B, c.H, c.T, c.D, c.W, alpha, f.f, f.K, c.dtype, &c.o, pw, nw, st);
+                     static_cast<float*>(pdd), c.B, c.H, c.T, c.D, c.W, alpha, f.f, f.K, c.dtype, &c.o, pw, nw, on.st);
     Py_END_ALLOW_THREADS
+    on.results({{&dq, own[0]}, {&dk, own[1]}, {&dv, own[2]}, {&dth, own[3]}, {&dd, own[4]}});
     if (rc) return PyLong_FromLong(rc);
     if (dth.defined() && !(dth.dim() == 1 && dth.size(0) == 1)) dth = dth.slice(0, 0, 1);
     if (dd.defined() && !(dd.dim() == 1 && dd.size(0) == f.K)) dd = dd.slice(0, 0, f.K);
