@@ -371,7 +371,8 @@ cudaError_t launch_nt(const BoxMaps& mq, const BoxMaps& mg, const BwdArgs& a, co
 }  // namespace
 
 size_t bwd_key_mma_static_smem() {
-    return sizeof(float) * (kWarps * kMmaMaxRungs * 16 + kWarps * 32 + kMmaMaxRungs) +
+    // rvals, wils, red, the RoPE steps; the barrier and alignment (rounded up)
+    return sizeof(float) * (kWarps * kMmaMaxRungs * 16 + kWarps * 32) + sizeof(double) * kMmaMaxRungs +
            sizeof(RopeSmem) + 64;
 }
 
