@@ -363,9 +363,8 @@ cudaError_t launch_nt(const BoxMaps& mq, const BoxMaps& mg, const BwdArgs& a, co
     const bool split = (long long)grid < 2LL * slots;
     auto kern = split ? bwd_key_mma_kernel<NT, true> : bwd_key_mma_kernel<NT, false>;
     if (split) grid *= 2;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_kernel(kern, dim3(grid), dim3(kWarps * 32), smem, st, mq, mg, a, L);
+    return launch_kernel_dynamic(kern, dim3(grid), dim3(kWarps * 32), smem, kBlockSmem - bwd_key_mma_static_smem(), st,
+                                 mq, mg, a, L);
 }
 
 }  // namespace

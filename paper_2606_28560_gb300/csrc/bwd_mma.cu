@@ -807,9 +807,8 @@ cudaError_t launch_nt(const RowMaps& mk, const RowMaps& mv, const QTileMaps& mt,
                       const MmaLayout& L, unsigned grid, size_t smem, cudaStream_t st) {
     auto kern = a.saved ? (a.want_dd ? bwd_query_mma_kernel<NT, true, true> : bwd_query_mma_kernel<NT, false, true>)
                         : (a.want_dd ? bwd_query_mma_kernel<NT, true, false> : bwd_query_mma_kernel<NT, false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_kernel(kern, dim3(grid), dim3(kWarps * 32), smem, st, mk, mv, mt, a, L);
+    return launch_kernel_dynamic(kern, dim3(grid), dim3(kWarps * 32), smem, kBlockSmem - bwd_mma_static_smem(), st, mk,
+                                 mv, mt, a, L);
 }
 
 }  // namespace

@@ -251,6 +251,19 @@ cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// The same with dynamic shared memory, `most` being the largest that any call
+// asks of this kernel.  The limit belongs to the function, and other host threads
+// launch it with other sizes at the same time: it is always set to `most`, so no
+// thread lowers it between another's set and launch.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_kernel_dynamic(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, size_t most,
+                                  cudaStream_t st, Args... args) {
+    if (smem > most) return cudaErrorInvalidValue;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    return e != cudaSuccess ? e : launch_kernel(kern, grid, block, smem, st, args...);
+}
+constexpr size_t kBlockSmem = 227 * 1024;         // shared memory of a block, static and dynamic
+
 // ----------------------------------------------------------- launchers ----
 
 cudaError_t launch_rope_rows(const void* src, void* dst, long long rows, int T, const RopeParams& rp,

@@ -602,9 +602,8 @@ cudaError_t launch_nt(const BoxMaps& mk, const BoxMaps& mv, const FwdArgs& a, co
                       unsigned grid, size_t smem, cudaStream_t st) {
     // (the grouped form runs only without residuals)
     auto kern = a.res_P ? fwd_mma_kernel<NT, TEAMS, TEAMS == 1> : fwd_mma_kernel<NT, TEAMS, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_kernel(kern, dim3(grid), dim3(kWarps * 32 * TEAMS), smem, st, mk, mv, a, L);
+    const size_t most = TEAMS == 1 ? kBlockSmem - fwd_mma_static_smem() : fwd_mma_gqa_smem_limit();
+    return launch_kernel_dynamic(kern, dim3(grid), dim3(kWarps * 32 * TEAMS), smem, most, st, mk, mv, a, L);
 }
 
 }  // namespace

@@ -864,10 +864,12 @@ size_t smem_of(bool split, size_t words) {
     return sizeof(float) * QW * (split ? kWarps * kHeadDim + words + kWarps : kWarps * words);
 }
 
-template <typename... KArgs, typename... Args>
-cudaError_t launch(void (*kern)(KArgs...), int grid, size_t smem, cudaStream_t st, const Args&... args) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return e != cudaSuccess ? e : launch_kernel(kern, dim3((unsigned)grid), dim3(kWarps * 32), smem, st, args...);
+// words(window slots of the table, rungs): the rows a kernel's table has.
+template <typename A, typename Words>
+cudaError_t launch(void (*kern)(A, RungList, int), int grid, bool split, Words words, cudaStream_t st, const A& a,
+                   const RungList& L, int chunk) {
+    return launch_kernel_dynamic(kern, dim3((unsigned)grid), dim3(kWarps * 32), smem_of(split, words(chunk, L.n)),
+                                 smem_of(split, words(kChunk, kMaxRungs)), st, a, L, chunk);
 }
 
 template <typename T>
@@ -877,7 +879,7 @@ cudaError_t launch_fwd(const FwdArgs& a, cudaStream_t st) {
     const bool split = split_rows(a.s, heads);
     auto kern = split ? fwd_gather_kernel<T, true, false>
                       : a.s.W + 1 > chunk ? fwd_gather_kernel<T, false, true> : fwd_gather_kernel<T, false, false>;
-    return launch(kern, blocks_of(a.s, heads), smem_of(split, chunk + L.n), st, a, L, chunk);
+    return launch(kern, blocks_of(a.s, heads), split, [](size_t w, size_t n) { return w + n; }, st, a, L, chunk);
 }
 
 template <typename T>
@@ -887,7 +889,8 @@ cudaError_t launch_query(const BwdArgs& a, cudaStream_t st) {
     const bool split = split_rows(a.s, heads), dd = a.want_dd;
     auto kern = split ? (dd ? bwd_query_gather_kernel<T, true, true> : bwd_query_gather_kernel<T, true, false>)
                       : (dd ? bwd_query_gather_kernel<T, false, true> : bwd_query_gather_kernel<T, false, false>);
-    return launch(kern, blocks_of(a.s, heads), smem_of(split, 2 * (chunk + L.n) + (dd ? 2 * L.n : 0) + 1), st, a, L, chunk);
+    return launch(kern, blocks_of(a.s, heads), split,
+                  [dd](size_t w, size_t n) { return 2 * (w + n) + (dd ? 2 * n : 0) + 1; }, st, a, L, chunk);
 }
 
 template <typename T>
@@ -896,7 +899,8 @@ cudaError_t launch_key(const BwdArgs& a, cudaStream_t st) {
     const int heads = a.s.B * a.s.Hkv, chunk = std::min(a.s.W + 1, kChunk);
     const bool split = split_rows(a.s, heads);
     auto kern = split ? bwd_key_gather_kernel<T, true> : bwd_key_gather_kernel<T, false>;
-    return launch(kern, blocks_of(a.s, heads) + (a.want_dd ? 1 : 0), smem_of(split, chunk + 2 * L.n), st, a, L, chunk);
+    return launch(kern, blocks_of(a.s, heads) + (a.want_dd ? 1 : 0), split,
+                  [](size_t w, size_t n) { return w + 2 * n; }, st, a, L, chunk);
 }
 
 }  // namespace
