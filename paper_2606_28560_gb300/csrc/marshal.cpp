@@ -44,6 +44,11 @@ double as_float(PyObject* o) {
     if (v == -1.0 && PyErr_Occurred()) throw python_error();
     return v;
 }
+bool as_bool(PyObject* o) {
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw python_error();
+    return v != 0;
+}
 
 // The base sequence: a C-contiguous float32 array (binding.py makes it one).
 struct Offsets {
@@ -86,8 +91,8 @@ struct Call {
         o = fibattn_opts{};
         o.rope_base = (float)as_float(a[0]);
         o.scale = (float)as_float(a[1]);
-        o.no_dedup = PyObject_IsTrue(a[2]) ? 0 : 1;
-        o.round_offsets = PyObject_IsTrue(a[3]) ? 1 : 0;
+        o.no_dedup = as_bool(a[2]) ? 0 : 1;
+        o.round_offsets = as_bool(a[3]) ? 1 : 0;
         o.Hkv = (int)k.size(1);
         o.rotated_k = ptr(rk);
         o.residuals = ptr(res);
@@ -260,6 +265,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     Call c(q, k, (int)as_int(a[4]), f, rk, res, a + 6);
     const float alpha = (float)as_float(a[5]);
     c.o.bwd_kernel = (int)as_int(a[10]);
+    const bool rung_grads = as_bool(a[23]);
     Tensor dq = optional(a[18], "dq"), dk = optional(a[19], "dk"), dv = optional(a[20], "dv");
     Tensor dth = optional(a[21], "dtheta"), dd = optional(a[22], "dd"), ws = optional(a[13], "workspace");
     check_kv(q, k, v);
@@ -277,7 +283,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const OnStream on(a[16]);
     const bool own[5] = {!dq.defined(), !dk.defined(), !dv.defined(), !dth.defined(), !dd.defined()};
     dq = like(dq, q); dk = like(dk, k); dv = like(dv, v);
-    if (PyObject_IsTrue(a[23])) {
+    if (rung_grads) {
         if (!dth.defined()) dth = at::empty({1}, q.options().dtype(at::kFloat));
         if (!dd.defined()) dd = at::empty({std::max(f.K, 1)}, q.options().dtype(at::kFloat));
     }
