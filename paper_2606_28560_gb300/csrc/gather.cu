@@ -238,7 +238,11 @@ struct Place {
     bool writer;                                  // one lane of the two
     int step, first;                              // batches: first, first + step, ...
     __device__ __forceinline__ Place(int tile) {
-        lane = threadIdx.x & 31; c = lane & 7; g = lane >> 3; warp = threadIdx.x >> 5;
+        lane = threadIdx.x & 31; c = lane & 7; g = lane >> 3;
+        // (through a shuffle, which makes it and all that follows from it uniform:
+        // with the bounds below the fp32 key pass spilled 128 bytes without it;
+        // layer B4 H8 T1000 W8 75.5 us without, 71.0 with)
+        warp = __shfl_sync(kAll, threadIdx.x >> 5, 0);
         iw = SPLIT ? tile * QW : (tile * kWarps + warp) * QW;
         row = iw + g * R + (c >> 1);
         writer = (c & 1) == 0;
@@ -249,6 +253,13 @@ struct Place {
         if (SPLIT) __syncthreads();
         else __syncwarp();
     }
+    // Window slots that any row of the warp has: as queries (slot t of query i is
+    // row i - t), as keys (slot t of query j + t reads key j).  A window longer
+    // than that is not walked: B4 H8 T128 W1024, fp32, forward 186 -> 30 us,
+    // backward 751 -> 88; B2 T2048 W1024 forward 495 -> 450, backward 2312 -> 1967.
+    // Slots beyond are in no table, nor in the workspace: no key has them either.
+    __device__ __forceinline__ int query_slots(const Shape& s) const { return min(s.W + 1, iw + QW); }
+    __device__ __forceinline__ int key_slots(const Shape& s) const { return min(s.W + 1, s.T - iw); }
 };
 template <bool SPLIT> constexpr int kTileRows16 = SPLIT ? QW : kWarps * QW;
 
@@ -468,9 +479,10 @@ __global__ void __launch_bounds__(kWarps * 32, MULTI ? 2 : 4) fwd_gather_kernel(
     const bool vo = p.row < s.T;
     float m = -INFINITY, l = 0.f;                             // of the lane's own row
 
-    for (int t0 = 0; t0 <= s.W; t0 += chunk) {
-        const int t1 = MULTI ? min(s.W + 1, t0 + chunk) : s.W + 1;
-        const bool last = !MULTI || t1 == s.W + 1;
+    const int slots = p.query_slots(s);
+    for (int t0 = 0; t0 < slots; t0 += chunk) {
+        const int t1 = MULTI ? min(slots, t0 + chunk) : slots;
+        const bool last = !MULTI || t1 == slots;
         const float m_old = m;
         // ---- scores of the chunk's window slots, and of the rungs at the end
         auto put = [&](int n, float sco) {
@@ -612,8 +624,9 @@ __global__ void __launch_bounds__(kWarps * 32, 4) bwd_query_gather_kernel(BwdArg
             }
         }
         if (sizeof(KT) == 2 && qmax >= 65520.f) raise_status(a.status, kStatusRange);   // fp16 rows hold < 65520
-        const int n_chunks = (s.W + chunk) / chunk;           // 1 with SPLIT
-        const int tl = (n_chunks - 1) * chunk, nw = s.W + 1 - tl;   // the last chunk's window slots
+        const int slots = p.query_slots(s);
+        const int n_chunks = (slots + chunk - 1) / chunk;     // 1 with SPLIT
+        const int tl = (n_chunks - 1) * chunk, nw = slots - tl;     // the last chunk's window slots
         // a chunk's table to the workspace, where it waits for Delta
         auto spill = [&](const float* tab, float* to, int t0) {
             __syncwarp();
@@ -621,8 +634,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4) bwd_query_gather_kernel(BwdArg
                 if (iq < s.T) to[(size_t)(t0 + u) * s.T + iq] = tab[u * QW + ql];
             __syncwarp();
         };
-        for (int t0 = 0; t0 <= s.W; t0 += chunk) {
-            dot_window(p, vec, Kt, s.T, t0, min(s.W + 1, t0 + chunk), [&](int t, float x) {
+        for (int t0 = 0; t0 < slots; t0 += chunk) {
+            dot_window(p, vec, Kt, s.T, t0, min(slots, t0 + chunk), [&](int t, float x) {
                 const float e = (vo && p.row >= t) ? prob(x) : 0.f;
                 if (p.writer) po[(t - t0) * QW] = e;
             });
@@ -651,9 +664,9 @@ __global__ void __launch_bounds__(kWarps * 32, 4) bwd_query_gather_kernel(BwdArg
 #pragma unroll
         for (int r = 0; r < R; ++r) load_row(dO + (size_t)min(p.iw + p.g * R + r, s.T - 1) * kHeadDim, p.c, vec[r]);
         float delta = 0.f;
-        for (int t0 = 0; t0 <= s.W; t0 += chunk) {
+        for (int t0 = 0; t0 < slots; t0 += chunk) {
             const bool here = t0 == tl;
-            dot_window(p, vec, V, s.T, t0, min(s.W + 1, t0 + chunk), [&](int t, float x) {
+            dot_window(p, vec, V, s.T, t0, min(slots, t0 + chunk), [&](int t, float x) {
                 const float dp = (vo && p.row >= t) ? x : 0.f;
                 const float e = here ? po[(t - t0) * QW] : vo ? Pg[(size_t)t * s.T + p.row] : 0.f;
                 delta = fmaf(e, dp, delta);
@@ -702,7 +715,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) bwd_query_gather_kernel(BwdArg
         // ---- dq~ += dS key rows
         float2 acc[R][4];
         clear(acc);
-        add_window(p, acc, Kt, s.T, tl, s.W + 1, dtab);
+        add_window(p, acc, Kt, s.T, tl, slots, dtab);
         add_rungs(p, acc, Kt, s.T, L, dtab + nw * QW);
         for (int ch = 0; ch + 1 < n_chunks; ++ch) {           // the earlier chunks, from the workspace
             const int t0 = ch * chunk, t1 = t0 + chunk;
@@ -761,6 +774,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) bwd_key_gather_kernel(BwdArgs 
     float* tab = SPLIT ? tab_all + kWarps * QW * kHeadDim : tab_all + (size_t)p.warp * ((chunk + 2 * L.n) * QW);
     float* tabg = tab + p.g * R;
     const int kl = p.lane & (QW - 1), sl = 2 * p.first + p.lane / QW;   // a lane's key and first slot in a sweep
+    const int slots = p.key_slots(s);
 
     // One output (dk~ from q~ rows and dS, then dv from dO rows and p) of the
     // warp's keys; weights: slot-major, S T values a head.
@@ -772,9 +786,9 @@ __global__ void __launch_bounds__(kWarps * 32, 4) bwd_key_gather_kernel(BwdArgs 
             const size_t bh = (size_t)b * s.H + hk * s.G + gq;
             const auto* base = rows + bh * s.T * kHeadDim;
             const float* Xh = weights + bh * a.S * s.T;
-            for (int t0 = 0; t0 <= s.W; t0 += chunk) {
-                const int t1 = min(s.W + 1, t0 + chunk), nw = t1 - t0;
-                const int nr = t1 == s.W + 1 ? L.n : 0;
+            for (int t0 = 0; t0 < slots; t0 += chunk) {
+                const int t1 = min(slots, t0 + chunk), nw = t1 - t0;
+                const int nr = t1 == slots ? L.n : 0;
                 // ---- the weights of the keys, all copies in flight together
                 for (int u = sl; u < nw + 2 * nr; u += 2 * p.step) {
                     const int rr = u - nw, n = rr >> 1;
