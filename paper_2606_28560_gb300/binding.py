@@ -101,6 +101,9 @@ def _marshal():
                 path = _build.MARSHAL
                 if not os.path.exists(path):
                     raise RuntimeError(f"native binding not built ({path} missing); run __graft_entry__.build()")
+                if not _build.marshal_fits():
+                    raise RuntimeError(f"native binding built for another PyTorch or Python ({path}); run "
+                                       "__graft_entry__.build()")
                 loader = importlib.machinery.ExtensionFileLoader("fibattn_marshal", path)
                 spec = importlib.util.spec_from_file_location("fibattn_marshal", path, loader=loader)
                 m = importlib.util.module_from_spec(spec)
