@@ -40,8 +40,11 @@ long as_int(PyObject* o) {
     return v;
 }
 double as_float(PyObject* o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw python_error();
+    if (PyFloat_CheckExact(o)) return PyFloat_AS_DOUBLE(o);
+    PyObject* const f = PyNumber_Float(o);        // what float() takes
+    if (!f) throw python_error();
+    const double v = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
     return v;
 }
 bool as_bool(PyObject* o) {
