@@ -82,10 +82,7 @@ __device__ __forceinline__ void key_pass(float (&acc)[8][4], const float* X, con
         const int i = u >> 4, x = u & 15;
         const int q = bw + L.act_s0[i] + x;
         const bool use = i < L.n_act && q < s.T;
-        // (NT = 4 from the host's row offsets, 94.9 -> 92.8 us at B2 T16384; the
-        // NT = 3 kernel is 1 % slower with them)
-        const unsigned row = NT == 4 ? (unsigned)L.act_row[i] : (unsigned)((s.W + 1 + L.act_k[i]) * s.T);
-        rvv[j] = use ? X[row + (unsigned)q] : 0.f;
+        rvv[j] = use ? X[(unsigned)((s.W + 1 + L.act_k[i]) * s.T + q)] : 0.f;
     }
     if (IL) {
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -265,10 +262,11 @@ bwd_key_mma_kernel(const __grid_constant__ BoxMaps tmQ, const __grid_constant__ 
             const float* X = (pass ? a.DSs : a.Ps) + (size_t)qhead * a.S * s.T;
             if (warp == 0) {
                 const BoxMaps& m = pass ? tmQ : tmG;
-                if (lane == 0) mbar_expect_tx(&bar, L.box_bytes);
+                if (lane == 0) {
+                    mbar_expect_tx(&bar, L.box_bytes);
+                    issue_boxes(sbase, m, L, j0, qhead, &bar);
+                }
                 __syncwarp();
-                if constexpr (NT == 4) issue_rows(sbase, m, L, j0, qhead, &bar, lane);
-                else if (lane == 0) issue_boxes(sbase, m, L, j0, qhead, &bar);
             }
             if (pass == 0)
                 key_pass<NT>(acc, X, a, L, sbase, bw, wrel, g4, c4, lane, vlo, vhi, &bar, parity, ok,

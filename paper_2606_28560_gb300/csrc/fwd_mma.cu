@@ -716,7 +716,7 @@ int interval_of(const MmaLayout& L, int smem_row) {
 
 // Active rungs sorted by d (ties by index), with their shared rows and the
 // merged interval of each slab.
-void active_list(const Shape& s, const RungParams& r, MmaLayout* L) {
+void active_list(const RungParams& r, MmaLayout* L) {
     L->n_act = 0;
     for (int i = 0; i < kMmaMaxRungs; ++i) {
         L->act_k[i] = 0; L->act_s0[i] = 0; L->act_smem[i] = 0; L->act_w[i] = 0.f; L->act_d[i] = 3.0e38f;
@@ -732,7 +732,6 @@ void active_list(const Shape& s, const RungParams& r, MmaLayout* L) {
         L->act_k[i] = k; L->act_s0[i] = r.s0[k]; L->act_smem[i] = L->rung_smem[k];
         L->act_w[i] = r.w[k]; L->act_d[i] = r.d[k];
     }
-    for (int i = 0; i < kMmaMaxRungs; ++i) L->act_row[i] = i < L->n_act ? (s.W + 1 + L->act_k[i]) * s.T : 0;
     for (int i = 0; i < kMmaMaxRungs; ++i) L->act_iv[i] = i < L->n_act ? interval_of(*L, L->act_smem[i]) : 0;
     L->win_iv = interval_of(*L, L->win_smem);
 }
@@ -794,7 +793,7 @@ bool build_mma_layout(const Shape& s, const RungParams& r, double rope_base, siz
     for (int k = 0; k < kMmaMaxRungs; ++k) L->rung_smem[k] = 0;
     for (int k = 0; k < r.K; ++k)
         if ((r.active >> k) & 1u) L->rung_smem[k] = smem_row_of(*L, -r.s0[k] - 1);
-    active_list(s, r, L);
+    active_list(r, L);
     L->buf_rows = L->rows;
     L->lo_start = 0;
     L->bytes_lo = (unsigned)L->rows * 128u;
@@ -822,7 +821,7 @@ bool build_key_layout(const Shape& s, const RungParams& r, double rope_base, siz
     for (int k = 0; k < kMmaMaxRungs; ++k) L->rung_smem[k] = 0;
     for (int k = 0; k < r.K; ++k)
         if ((r.active >> k) & 1u) L->rung_smem[k] = smem_row_of(*L, r.s0[k]);
-    active_list(s, r, L);
+    active_list(r, L);
     L->buf_rows = L->rows;
     L->lo_start = 0;
     L->bytes_lo = (unsigned)L->rows * 128u;

@@ -33,7 +33,6 @@ struct MmaLayout {
     int act_smem[kMmaMaxRungs];
     float act_w[kMmaMaxRungs];
     float act_d[kMmaMaxRungs];
-    int act_row[kMmaMaxRungs];                    // (W + 1 + k) T: the rung's row of a head's slot-major arrays
     int act_iv[kMmaMaxRungs];                     // merged interval that holds the rung's slab
     int win_iv;                                   // merged interval that holds the window band
     // Staging buffer rows (>= rows).  A kernel that first copies its tile's own

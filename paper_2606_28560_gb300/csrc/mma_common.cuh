@@ -153,21 +153,24 @@ __device__ __forceinline__ unsigned row_chunk(unsigned base, int row, int ch) {
 // go out one after another, so they are few: per merged interval whole 64-row
 // boxes, and for the rest of it one box of 32 or 64 rows that ends with the
 // interval and repeats rows of the box before (8-row boxes made up to seven of
-// that rest).  Forward B4 T4096 W10 40.5 -> 38.4 us a call; training layer B16
-// T1024 133.6 -> 131.7, with two kv heads 127.1 -> 124.2, B2 T16384 pow2 227.7
-// -> 223.4.  Two forms, for kernels that the compiler schedules differently
-// around them (NT = 4 with residuals: 84.3 us lane by lane, 88.3 from the list;
-// NT = 3 without: 39.7 and 37.2; issued by all eight warps: slower than by
-// one).  Both deliver L.box_bytes, with which somebody arms the barrier in the
-// same phase.
+// that rest): forward B4 T4096 W10 40.9 -> 38.8 us, with residuals B16 T1024 W8
+// 45.3 -> 43.3, key pass 48.5 -> 47.2 there.  Issued by all eight warps: slower
+// than by one.  Both forms deliver L.box_bytes, with which somebody arms the
+// barrier in the same phase.
 //
-// issue_boxes: one thread, from the host's flat list.
+// issue_boxes: one thread, from the host's flat list.  All kernels but the one
+// below; lane by lane against it (B16 T1024): forward W0 43.0 / 42.9 us, W8 37.8 /
+// 37.1, W12 37.3 / 35.3, W16 37.9 / 35.5, with residuals W0 51.7 / 51.5, W8
+// 44.7 / 43.3; key pass B2 T16384 W12 84.7 / 83.9, W16 87.6 / 85.8, W8 as fast.
 __device__ __forceinline__ void issue_boxes(unsigned dst, const BoxMaps& m, const MmaLayout& L, int i0, int head,
                                             unsigned long long* bar) {
     for (int b = 0; b < L.n_box; ++b)
         tma_load_3d(dst + (unsigned)L.box_smem[b] * 128u, b < L.n_box64 ? &m.m64 : &m.m32, 0, i0 + L.box_row[b], head, bar);
 }
-// issue_rows: one warp, lane n copies merged interval n.
+// issue_rows: one warp, lane n copies merged interval n.  The NT = 4 forward with
+// residuals (W 9 .. 16), which the compiler schedules better around it: B2 T16384
+// W12 84.4 us, from the list 88.5, W16 82.4 and 86.3 (power-of-2 rungs 65.9 and
+// 69.1); at B16 T1024 44.8 and 45.3.
 __device__ __forceinline__ void issue_rows(unsigned dst, const BoxMaps& m, const MmaLayout& L, int i0, int head,
                                            unsigned long long* bar, int lane) {
     for (int iv = lane; iv < L.n_iv; iv += 32) {
