@@ -64,9 +64,9 @@ __global__ void __launch_bounds__(256, 4) rope_rows_bf16_kernel(const __nv_bfloa
         const float2* cp = reinterpret_cast<const float2*>(ctab + pr * kRopeTabStride + 8 * c);
         const float2* sp = reinterpret_cast<const float2*>(stab + pr * kRopeTabStride + 8 * c);
         // The thread's items share their position.  With two items their angles,
-        // read once, fit the 64 registers (layer B2 H8 T16384 forward + backward
-        // 271.7 -> 271.2 us, power-of-2 base 214.7 -> 214.0); with four they spill
-        // (forward B16 H8 T1024 38.0 -> 41.0 us).
+        // read once, fit the 64 registers (B2 H8 T16384: this kernel 16.7 -> 16.1 us,
+        // a layer's forward and backward 305.9 -> 304.6 at W 0, 274.0 -> 273.4 at W 8);
+        // with four they spill (forward B16 H8 T1024 38.0 -> 41.0 us).
         constexpr bool kKeep = kItems <= 2;
         float2 cv[4], sv[4];
 #pragma unroll
