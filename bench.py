@@ -268,15 +268,15 @@ def step_method_bytes():
 # lines only: comments and blank lines are left out): once the code of a file
 # of the kernel changes, the figure is reported as null until the next capture.
 NCU_TRAFFIC = {
-    "bwd_query_mma": {"bytes_at_b32": 165826560 + 34649856,
+    "bwd_query_mma": {"bytes_at_b32": 165826304 + 34677504,
                       "sources": ("bwd_mma.cu", "mma_common.cuh", "fwd_mma.cuh", "fibattn_internal.cuh"),
-                      "sha256": "21821344fbc102b8f92e80482f8298a1532983e746753a7c0afda5a66c384805"},
-    "bwd_key_mma": {"bytes_at_b32": 104474112 + 36254464,
+                      "sha256": "7a6eb2f7d4feb3df5fe17da5c123412960a0f981820708d5c6c8d90417a9135f"},
+    "bwd_key_mma": {"bytes_at_b32": 104474112 + 36588544,
                     "sources": ("bwd_key_mma.cu", "mma_common.cuh", "fwd_mma.cuh", "fibattn_internal.cuh"),
-                    "sha256": "765280ce807e12c46e3220248e7348fa6ab252fc81245b85f9100b562971ea78"},
-    "fwd": {"bytes_at_b32": 100809216 + 57611264,
+                    "sha256": "4ff4e27482277785ddef47bd09570cc27c9726b314342d7705918d65cdc68e90"},
+    "fwd": {"bytes_at_b32": 100786432 + 57735424,
             "sources": ("fwd_mma.cu", "mma_common.cuh", "fwd_mma.cuh", "fibattn_internal.cuh"),
-            "sha256": "0924d8b3132882c710ecea13e495835180fd9a518aa9aa5d5fe907f97b44bf4a"},
+            "sha256": "f5e65c2459e7c5aefee87e45327bf46bd1462355ff93fb85501562b94d5cc0c5"},
 }
 
 
@@ -902,28 +902,33 @@ def ncu_case(which: str):
     path the bench times: the forward keeps its rotated keys and residuals,
     the backward reads them (per layer and pass: RoPE of k, forward, query
     pass, key pass).  `fwd_plain`: the forward alone without residuals (the
-    forward-only workload, alpha 0.9 in both layers)."""
+    forward-only workload, alpha 0.9 in both layers).  `fp32`: forward and
+    backward with fp32 I/O (the row-gather kernels), B=16, alpha 0.9 (the same
+    bytes a layer)."""
     import __graft_entry__
     __graft_entry__.build()
     import paper_2606_28560_gb300 as fa
     from paper_2606_28560_gb300 import inputs
     dev = torch.device("cuda", 0)
-    Bc, layers = 32, 2
+    fp32 = which == "fp32"
+    Bc, layers = 16 if fp32 else 32, 2
+    dtype = torch.float32 if fp32 else torch.bfloat16
     f = fa.base("fib", K)
     bufs = []
     for l in range(layers):
-        ts = [torch.empty((Bc, H, T, D), dtype=torch.bfloat16, device=dev) for _ in range(4)]
+        ts = [torch.empty((Bc, H, T, D), dtype=dtype, device=dev) for _ in range(4)]
         for j, t in enumerate(ts):
             inputs.device_normal_(t, 1000 + 10 * l + j)
-        bufs.append(ts + [fa.residuals_like(ts[0], W, K), fa.rotated_k_like(ts[1])])
+        bufs.append(ts + [None if fp32 else fa.residuals_like(ts[0], W, K), fa.rotated_k_like(ts[1])])
     for rep in range(2):
         for l, (q, k, v, g, res, rk) in enumerate(bufs):
             if which == "fwd_plain":
                 fa.fwd(q, k, v, 0.9, f, W, rotated_k=rk)
                 continue
-            out, lse = fa.fwd(q, k, v, 0.8 + 0.1 * l, f, W, residuals=res, rotated_k=rk)
-            if which == "bwd":
-                fa.bwd(q, k, v, lse, g, 0.8 + 0.1 * l, f, W, out=out, residuals=res, rotated_k=rk)
+            alpha = 0.9 if fp32 else 0.8 + 0.1 * l
+            out, lse = fa.fwd(q, k, v, alpha, f, W, residuals=res, rotated_k=rk)
+            if which != "fwd":
+                fa.bwd(q, k, v, lse, g, alpha, f, W, out=out, residuals=res, rotated_k=rk)
     torch.cuda.synchronize(dev)
     print(f"ncu case {which} done")
 
@@ -937,7 +942,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=10)
     ap.add_argument("--impl", default="gb300", choices=["gb300", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--ncu-case", choices=["fwd", "fwd_plain", "bwd"], default=None,
+    ap.add_argument("--ncu-case", choices=["fwd", "fwd_plain", "bwd", "fp32"], default=None,
                     help="run a small fixed case for an ncu capture and exit")
     args = ap.parse_args()
     if args.ncu_case:

@@ -20,15 +20,27 @@
 // block take the same 16 rows and share out the window rows and the rungs; the
 // table is then the block's, and the four partial sums meet in shared memory.
 //
-// Bound by load latency and issue, not bytes: 120-128 registers leave 16 warps
-// an SM, issue is active 40 % of cycles, L1 50 %.  Against one 4-lane group a
-// row that walked its slots one after another (graph-replayed, us):
-//   fp32 W 8 B4 H8 T1000   forward 34.5 -> 25.1, query pass with the rotation of
-//                          q 58 -> 38.7, key pass 61 -> 24.9, layer 142.6 -> 75.8
-//   fp32 W 8 B16 H8 T1024  forward 105.8 -> 63;  B1: call 12.9 -> 11.4
-//   bf16 W 32 B4 H8 T1024  35.8 -> 31.3, 65 -> 48.9, 67 -> 29.3, layer 153.7 -> 96.1
-//   bf16 W 200 B2 H8 T1000 layer 400 -> 260
-// (Two rows a group: layer 118 us; two or eight warps a block: 93 us and worse.)
+// Bound by load latency and issue, not bytes: 113-128 registers leave 16 warps
+// an SM at the narrow windows of the paper; the query pass's tables (a quarter KB
+// a block for each 2 W + 13 + 2 rungs) leave 12 from W of about 100 on, 8 from 140,
+// and 4 at W 207 with 15 rungs beyond it.  Issue is active 44-47 % of cycles, L1
+// 56-60 % (fp32 B16 T1024 W 8).  Against one 4-lane group a row that
+// walked its slots one after another (us):
+//   fp32 W 8 B4 H8 T1000   forward 34.5 -> 24.5, query pass with the rotation of
+//                          q 58 -> 36.6, key pass 61 -> 24.4
+//   fp32 W 8 B16 H8 T1024  forward 105.8 -> 61.4
+//   bf16 W 32 B4 H8 T1024  35.8 -> 30.3, 65 -> 46.8, 67 -> 28.5
+// and graph-replayed, forward and backward: bf16 W 200 B2 H8 T1000 400 -> 245,
+// W 1024 B2 H8 T2048 2717 -> 2259, W 300 B4 H8 T4096 2681 -> 2147.
+// (Two rows a group: layer 118 us for the 73.8 of fp32 B4 T1000; two or eight
+// warps a block: 93 us and worse.)
+//
+// kChunk, the most window slots a table holds: wider windows pay for passes over
+// the table, and narrower ones that would fit must not.  104: fp32 B4 T1000 W150
+// forward 61.7 -> 83.4 us, W200 76.5 -> 103; but with more warps an SM the backward
+// of W300 B4 T4096 takes 1444 instead of 1789.  312: W 208 to 311 gain up to a
+// fifth in the backward (253 -> 204 at B2 T1000 W208), wider ones lose up to half
+// (W300 B4 T4096, a table 1.4 times as large: 1789 -> 2439).
 #include <algorithm>
 #include <cstring>
 #include <type_traits>
