@@ -268,9 +268,10 @@ struct Place {
     // Window slots that any row of the warp has: as queries (slot t of query i is
     // row i - t), as keys (slot t of query j + t reads key j).  A window longer
     // than that is not walked: B4 H8 T128 W1024, fp32, forward 186 -> 30 us,
-    // backward 751 -> 88; B2 T2048 W1024 forward 495 -> 450, backward 2312 -> 1967.
+    // backward 751 -> 88 (13 and 39 with tables for the sequence, see window_slots);
+    // B2 T2048 W1024 forward 495 -> 443, backward 2312 -> 1953.
     // Slots beyond are in no table, nor in the workspace: no key has them either.
-    __device__ __forceinline__ int query_slots(const Shape& s) const { return min(s.W + 1, iw + QW); }
+    __device__ __forceinline__ int query_slots(const Shape& s) const { return min(min(s.W + 1, s.T), iw + QW); }
     __device__ __forceinline__ int key_slots(const Shape& s) const { return min(s.W + 1, s.T - iw); }
 };
 template <bool SPLIT> constexpr int kTileRows16 = SPLIT ? QW : kWarps * QW;
@@ -870,13 +871,19 @@ __global__ void __launch_bounds__(kWarps * 32, 4) bwd_key_gather_kernel(BwdArgs 
 
 // ------------------------------------------------------------ host side ----
 
+// Window slots that any row has.  Tables are made for these, not for the window,
+// and so is the choice of the kernel: at T 20 and W 1024 (fp32 B64 H16 Hkv2) tables
+// of kChunk slots left one block an SM, forward 34.5 us, backward 114.7; now 15.7
+// and 62.1.  B4 H8 T128 W1024, whose rows are now shared: 30 -> 13 us, 88 -> 39.
+int window_slots(const Shape& s) { return std::min(s.W + 1, s.T); }
+
 // Whether the warps of a block share their rows: while the blocks that takes
 // all fit the GPU at once (four on each of 152 SMs; a constant, because the
 // size of the workspace depends on it).  A training layer (fp32, W 8, H 8,
 // T 1000) split / not: B1, 504 blocks, 36 / 56 us; B2, 1008 blocks, 62.9 /
 // 66.8 us, but its key pass 22.5 / 18.6 us; B3, 1512 blocks, 86.9 / 73.7 us.
 bool split_rows(const Shape& s, int heads) {
-    return s.W + 1 <= kChunk && (long long)((s.T + QW - 1) / QW) * heads <= 4 * 152;
+    return window_slots(s) <= kChunk && (long long)((s.T + QW - 1) / QW) * heads <= 4 * 152;
 }
 
 int blocks_of(const Shape& s, int heads) {
@@ -901,17 +908,17 @@ cudaError_t launch(void (*kern)(A, RungList, int), int grid, bool split, Words w
 template <typename T>
 cudaError_t launch_fwd(const FwdArgs& a, cudaStream_t st) {
     const RungList L = rung_list(a.r);
-    const int heads = a.s.B * a.s.H, chunk = std::min(a.s.W + 1, kChunk);
+    const int heads = a.s.B * a.s.H, chunk = std::min(window_slots(a.s), kChunk);
     const bool split = split_rows(a.s, heads);
     auto kern = split ? fwd_gather_kernel<T, true, false>
-                      : a.s.W + 1 > chunk ? fwd_gather_kernel<T, false, true> : fwd_gather_kernel<T, false, false>;
+                      : window_slots(a.s) > chunk ? fwd_gather_kernel<T, false, true> : fwd_gather_kernel<T, false, false>;
     return launch(kern, blocks_of(a.s, heads), split, [](size_t w, size_t n) { return w + n; }, st, a, L, chunk);
 }
 
 template <typename T>
 cudaError_t launch_query(const BwdArgs& a, cudaStream_t st) {
     const RungList L = rung_list(a.r);
-    const int heads = a.s.B * a.s.H, chunk = std::min(a.s.W + 1, kChunk);
+    const int heads = a.s.B * a.s.H, chunk = std::min(window_slots(a.s), kChunk);
     const bool split = split_rows(a.s, heads), dd = a.want_dd;
     auto kern = split ? (dd ? bwd_query_gather_kernel<T, true, true> : bwd_query_gather_kernel<T, true, false>)
                       : (dd ? bwd_query_gather_kernel<T, false, true> : bwd_query_gather_kernel<T, false, false>);
@@ -922,7 +929,7 @@ cudaError_t launch_query(const BwdArgs& a, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_key(const BwdArgs& a, cudaStream_t st) {
     const RungList L = rung_list(a.r);
-    const int heads = a.s.B * a.s.Hkv, chunk = std::min(a.s.W + 1, kChunk);
+    const int heads = a.s.B * a.s.Hkv, chunk = std::min(window_slots(a.s), kChunk);
     const bool split = split_rows(a.s, heads);
     auto kern = split ? bwd_key_gather_kernel<T, true> : bwd_key_gather_kernel<T, false>;
     return launch(kern, blocks_of(a.s, heads) + (a.want_dd ? 1 : 0), split,

@@ -78,3 +78,17 @@ def test_a_longer_window_costs_no_more_than_the_sequence():
         fa.fwd(q, k, v, 0.9, F, W, out=out, lse=lse, workspace=ws)
         fa.bwd(q, k, v, lse, g, 0.9, F, W, workspace=ws)
     assert _us(lambda: layer(1024)) <= 3 * _us(lambda: layer(127))
+
+
+def test_tables_are_made_for_the_sequence():
+    """The same at T = 20, where tables of 208 slots left one block an SM: three
+    times W = 19's time; now the two take the same kernels and sizes."""
+    B, H, T = 64, 16, 20
+    q, k, v, g = (x.cuda() for x in inputs.qkv(B, H, T, seed=1) + (inputs.dout(B, H, T, seed=2),))
+    ws = torch.empty(fa.bwd_workspace_bytes(B, H, T, 1024, len(F), torch.float32), dtype=torch.uint8, device="cuda")
+    out, lse = fa.fwd(q, k, v, 0.9, F, 19)
+
+    def layer(W):
+        fa.fwd(q, k, v, 0.9, F, W, out=out, lse=lse, workspace=ws)
+        fa.bwd(q, k, v, lse, g, 0.9, F, W, workspace=ws)
+    assert _us(lambda: layer(1024)) <= 1.5 * _us(lambda: layer(19))
