@@ -67,7 +67,7 @@ def _attend(q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha):
     alpha = None if alpha is None else float(alpha)
     if (torch.is_grad_enabled() and (q.requires_grad or k.requires_grad or v.requires_grad or theta.requires_grad)) \
             or torch._C._are_functorch_transforms_active() or torch.autograd.forward_ad._current_level >= 0 \
-            or torch.jit.is_tracing():
+            or torch._C._is_tracing():
         return FibAttentionFunction.apply(q, k, v, theta, offsets, W, rope_base, scale, dedup, alpha)
     if alpha is None:
         alpha = alpha_of_theta(float(theta))

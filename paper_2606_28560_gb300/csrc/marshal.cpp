@@ -133,6 +133,15 @@ Tensor bytes(size_t need, const Tensor& q) {
     return at::empty({(int64_t)std::max<size_t>(need, 256)}, q.options().dtype(at::kByte));
 }
 
+// The device of a call is that of its tensors.  (A plain guard asks the runtime
+// for the current device at both ends.)
+struct OnDevice {
+    c10::cuda::OptionalCUDAGuard guard;
+    explicit OnDevice(const Tensor& q) {
+        if (c10::cuda::current_device() != q.device().index()) guard.set_device(q.device());
+    }
+};
+
 // The stream of a call: the current one, or the caller's.  Memory allocated
 // while it stands comes from that stream's pool: a workspace released on return
 // is reused by later work of the same stream only, where the current stream's
@@ -141,7 +150,8 @@ struct OnStream {
     const c10::cuda::CUDAStream current;
     cudaStream_t st;
     c10::cuda::OptionalCUDAStreamGuard guard;
-    explicit OnStream(PyObject* o) : current(c10::cuda::getCurrentCUDAStream()), st(current.stream()) {
+    OnStream(PyObject* o, const Tensor& q)
+        : current(c10::cuda::getCurrentCUDAStream(q.device().index())), st(current.stream()) {
         if (o == Py_None) return;
         st = static_cast<cudaStream_t>(PyLong_AsVoidPtr(o));
         if (!st && PyErr_Occurred()) throw python_error();
@@ -208,8 +218,8 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_buffer(lse, q, at::kFloat, q.size(0) * q.size(1) * q.size(2), "lse");
     check_workspace(ws, q);
     check_inputs(q, {&q, &k, &v}, kFwdInputs);
-    const c10::cuda::CUDAGuard device(q.device());
-    const OnStream on(a[16]);
+    const OnDevice device(q);
+    const OnStream on(a[16], q);
     const Tensor out = like(given, q);
     const bool own_lse = !lse.defined();
     if (!lse.defined()) lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
@@ -232,12 +242,12 @@ PyObject* fwd_keep(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const float alpha = (float)as_float(a[5]);
     check_kv(q, k, v);
     check_inputs(q, {&q, &k, &v}, kFwdInputs);
-    const c10::cuda::CUDAGuard device(q.device());
+    const OnDevice device(q);
     const Tensor out = at::empty(q.sizes(), q.options());
     const Tensor lse = at::empty({c.B, c.H, c.T}, q.options().dtype(at::kFloat));
     const Tensor rk = at::empty(k.sizes(), k.options().dtype(c.dtype == FIBATTN_BF16 ? at::kHalf : at::kFloat));
     c.o.rotated_k = ptr(rk);
-    void* const st = c10::cuda::getCurrentCUDAStream().stream();
+    void* const st = c10::cuda::getCurrentCUDAStream(q.device().index()).stream();
     const size_t nr = fibattn_residual_bytes(c.B, c.H, c.T, c.D, c.W, f.K, c.dtype);
     Tensor res;
     int rc = FIBATTN_ERR_UNSUPPORTED;
@@ -282,8 +292,8 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_buffer(dd, q, at::kFloat, f.K, "dd");
     check_workspace(ws, q);
     check_inputs(q, {&q, &k, &v, &dout, &out}, "q, k, v, dout, out must be contiguous CUDA tensors of one dtype");
-    const c10::cuda::CUDAGuard device(q.device());
-    const OnStream on(a[16]);
+    const OnDevice device(q);
+    const OnStream on(a[16], q);
     const bool own[5] = {!dq.defined(), !dk.defined(), !dv.defined(), !dth.defined(), !dd.defined()};
     dq = like(dq, q); dk = like(dk, k); dv = like(dv, v);
     if (rung_grads) {
